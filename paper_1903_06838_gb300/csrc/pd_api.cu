@@ -586,6 +586,7 @@ int create_impl(const pd_geometry* geometry, uint32_t n_gains, uint32_t gain_shi
         }
     }
     c->masked = masked;
+    p.mean_frac = g.cm_mode >= PD_CM_MEAN && !ag ? pd::mean_frac_bits(p, pedestal_host) : -1;
     cudaError_t e;
     std::vector<float> nped(fpx);
     for (size_t i = 0; i < fpx; i++) nped[i] = -pedestal_host[i];

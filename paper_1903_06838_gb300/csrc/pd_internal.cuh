@@ -28,6 +28,9 @@ struct ChainParams {
     float cm_cut, zero_thr, seed_thr, photon_kev;
     float hist_inv_w, hist_neg_lo_s;  // bin(v) = floor(fma(v, inv_w, neg_lo_s))
     uint32_t hist_bins;
+    // mean common mode: binary places of every d = raw - pedestal when one
+    // pass of integer sums is exact (mean_frac_bits), else -1
+    int mean_frac;
     // device state owned by the context
     const float* ped;           // [frame_px]
     const float* nped;          // [frame_px] -pedestal (d = raw + nped)
@@ -155,6 +158,7 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
                            const CallOut& out, cudaStream_t stream,
                            const MultiGain* mg = nullptr);
 // The paper's mean estimator, one stage or three stacked (pd_cm_mean.cu).
+int mean_frac_bits(const ChainParams& p, const float* pedestal);
 cudaError_t launch_cm_mean(const ChainParams& p, const uint16_t* raw, uint32_t n_frames,
                            float* cm, cudaStream_t stream);
 
