@@ -262,7 +262,7 @@ cudaError_t launch_stencil_for(const pd_ctx* c, const uint16_t* fr, uint32_t nf,
     if (c->use_lean && c->kernels == 1) {
         pd::LeanConfig lc = c->lean_cfg;
         lc.wait_polls = c->wait_polls;
-        return pd::launch_stencil_lean(c->params, lc, fr, nf, frame_base, co, c->d_err, s);
+        return pd::launch_stencil_lean(c->params, lc, fr, nf, frame_base, co, c->d_err, s, mg);
     }
     return c->use_band
                ? pd::launch_stencil_band(c->params, c->band_cfg, fr, nf, frame_base, co, s, mg)
@@ -274,15 +274,15 @@ cudaError_t launch_cm(const pd_ctx* c, const uint16_t* fr, uint32_t nf, float* c
                       cudaStream_t s) {
     if (pd::cm_kind(c->params) == PD_CM_MEAN || pd::cm_kind(c->params) == PD_CM_MEAN_STACKED)
         return pd::launch_cm_mean(c->params, fr, nf, cm, s);
-    if (c->multigain)
-        return c->use_cm_big ? pd::launch_cm_big(c->params, c->cm_cfg, fr, nf, cm, s,
-                                                 ~c->mg.vmask & 0xFFFFu)
-                             : pd::launch_cm_select(c->params, fr, nf, cm, s, &c->mg);
     if (c->use_bank && c->kernels == 1) {
         pd::CodeMap cmap = c->cmap;
         cmap.wait_polls = c->wait_polls;
         return pd::launch_cm_bank(c->params, c->cm_cfg, cmap, fr, nf, cm, c->d_err, s);
     }
+    if (c->multigain)
+        return c->use_cm_big ? pd::launch_cm_big(c->params, c->cm_cfg, fr, nf, cm, s,
+                                                 ~c->mg.vmask & 0xFFFFu)
+                             : pd::launch_cm_select(c->params, fr, nf, cm, s, &c->mg);
     return c->use_cm_big    ? pd::launch_cm_big(c->params, c->cm_cfg, fr, nf, cm, s)
            : c->use_cm_rows ? pd::launch_cm_rows(c->params, fr, nf, cm, s)
                             : pd::launch_cm_select(c->params, fr, nf, cm, s);
@@ -651,15 +651,21 @@ int create_impl(const pd_geometry* geometry, uint32_t n_gains, uint32_t gain_shi
         // and the one-kernel chain read single-gain words
         c->use_cm_rows = c->use_fused = false;
         c->use_band = c->use_band && c->band_cfg.vec == 4;
-    } else if (!ag) {
-        // the lean pair: single-gain words, common mode before gain
-        c->lean_cfg = pd::make_lean_config(p);
-        c->use_lean = c->lean_cfg.ok &&
-                      (g.cm_mode == PD_CM_MEDIAN || g.cm_mode == PD_CM_NONE || g.cm_mode == PD_CM_MEAN);
+    }
+    if (!ag) {
+        // the lean pair: common mode before gain
+        c->lean_cfg = pd::make_lean_config(p, 0, c->multigain);
+        c->use_lean = c->lean_cfg.ok;
         std::vector<uint16_t> km;
         pd::CodeMap cmap{};
+        // Auto-ranging words outside stage 0 are at least 2^gain_shift.  Where
+        // the raw cap lies no higher, they take the code of a word at the cap,
+        // the spare bin of d >= cut, and the whole-unit selection's d (stage
+        // 0's pedestal) is past the cut too: the bank median reads them as it
+        // reads single-gain words (64 frames of 32 x 185 x 388: 257 us with the
+        // floating-point bank median, 222 us).
         if (c->use_cm_big && pd::build_code_map(p, pedestal_host, &km, &cmap) &&
-            pd::cm_bank_supported(p, cmap)) {
+            pd::cm_bank_supported(p, cmap) && (!n_gains || cmap.rcap <= (1u << gain_shift))) {
             if ((e = cudaMalloc(&c->d_kmap, km.size() * 2)) != cudaSuccess) {
                 free_ctx(c);
                 return fail(PD_ENOMEM, "device allocation failed in pd_create");
@@ -671,7 +677,8 @@ int create_impl(const pd_geometry* geometry, uint32_t n_gains, uint32_t gain_shi
             cmap.kmap = c->d_kmap;
             c->cmap = cmap;
             c->use_bank = true;
-            c->use_queue = c->use_lean && pd::queue_supported(p, cmap, c->lean_cfg);
+            c->use_queue =
+                c->use_lean && !c->multigain && pd::queue_supported(p, cmap, c->lean_cfg);
         }
     }
     pd::noalloc_prepare(c->device);
@@ -928,7 +935,7 @@ int pd_set_tuning(pd_ctx* c, const pd_tuning* t) {
     if (t->kernels > 3) return fail(PD_EINVAL, "kernels is 0, 1, 2 or 3");
     if (t->kernels) c->kernels = t->kernels;
     if (t->band_rows && c->use_lean) {
-        const pd::LeanConfig lc = pd::make_lean_config(c->params, t->band_rows);
+        const pd::LeanConfig lc = pd::make_lean_config(c->params, t->band_rows, c->multigain);
         if (!lc.ok || lc.rb != std::min(t->band_rows, c->params.rows))
             return fail(PD_EINVAL, "band too tall for shared memory");
         c->lean_cfg = lc;

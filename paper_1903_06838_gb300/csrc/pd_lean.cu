@@ -519,10 +519,18 @@ __global__ void __launch_bounds__(kBankThreads, 2)
 // Lean stencil over bands of full-width rows.
 constexpr uint32_t kLeanThreads = 512;
 
+// What a lean stencil instance handles beside the plain energies (64 frames
+// of 32 x 185 x 388, against the band stencil of pd_fast.cu that ran them
+// before: stacked 362 -> 272 us, auto-ranging 448 -> 371 us).
+constexpr int kPlain = 0;
+constexpr int kStacked = 1;    // the stacked mean's module-row and module-column terms
+constexpr int kMultiGain = 2;  // auto-ranging words
+
 struct LeanRow {
     uint2 rw;   // four raw words
     float4 np;  // their negated pedestals
     float4 g;   // their inverse gains
+    float cr;   // negated module-row term (kStacked)
 };
 
 // Shared memory of the lean stencil: the staged raw rows (STAGE), the tile
@@ -572,9 +580,11 @@ __device__ __forceinline__ LeanLane lean_lane(const ChainParams& p, const LeanCo
 // with rowlane false own no rows (blocks larger than tx * ty).
 // issue_next() runs on thread 0 once the stage is read.  False if a staged
 // copy's wait gave up.  ONEUNIT (per-row table only): every four-pixel chunk
-// lies inside one common-mode unit (unit_cols a multiple of 4).
-template <bool COLBANK, bool CORR, bool STAGE, bool ONEUNIT, class NextFn>
-__device__ __forceinline__ bool lean_tile(const ChainParams& p, const uint16_t* __restrict__ raw,
+// lies inside one common-mode unit (unit_cols a multiple of 4).  EXTRA:
+// kPlain, kStacked or kMultiGain (mg).
+template <bool COLBANK, bool CORR, bool STAGE, bool ONEUNIT, int EXTRA, class NextFn>
+__device__ __forceinline__ bool lean_tile(const ChainParams& p, const MultiGain& mg,
+                                          const uint16_t* __restrict__ raw,
                                           uint32_t frame_base, const CallOut& out,
                                           const LeanConfig& lc, const LeanSmem& sm,
                                           const LeanLane& L, uint32_t f, uint32_t m, uint32_t band,
@@ -611,7 +621,18 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const uint16_t* 
         const uint16_t* fr = raw + (size_t)f * p.frame_px + mod_base;
         const float* npm = p.nped + mod_base;
         const float* gm = p.inv_gain + mod_base;
-        const float* cmf = out.cm + (size_t)f * p.units_per_frame + (size_t)m * p.units_per_module;
+        const float* cm_frame =
+            out.cm + (size_t)f * (EXTRA == kStacked ? cm_per_frame(p) : p.units_per_frame);
+        const float* cmf = cm_frame + (size_t)m * p.units_per_module;
+        // kStacked: the module's row terms, and the chunk's four column terms
+        const float* cmr = cm_frame + p.units_per_frame + (size_t)m * p.rows;
+        float2 cc01 = make_float2(0.0f, 0.0f), cc23 = cc01;
+        if (EXTRA == kStacked) {
+            const float* cmc = cm_frame + p.units_per_frame + (size_t)p.n_modules * p.rows +
+                               (size_t)m * p.cols + col;
+            cc01 = make_float2(-__ldg(cmc), -__ldg(cmc + 1));
+            cc23 = make_float2(-__ldg(cmc + 2), -__ldg(cmc + 3));
+        }
         // stage row of module row r: r + srow0
         const int srow0 =
             STAGE ? (int)(m * p.rows) - (((int)(m * p.rows) + r0 - 1) & ~(int)(T - 1)) : 0;
@@ -657,7 +678,7 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const uint16_t* 
             __syncthreads();
         }
 
-        // e of four pixels of module row r, from a row of loads
+        // e of four pixels of the module row at tile row rl, from a row of loads
         auto correct = [&](const LeanRow& x, int rl, float2& e01, float2& e23) {
             const float2 d01 = __fadd2_rn(raw_pair(x.rw.x), make_float2(x.np.x, x.np.y));
             const float2 d23 = __fadd2_rn(raw_pair(x.rw.y), make_float2(x.np.z, x.np.w));
@@ -672,8 +693,36 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const uint16_t* 
                 m01 = make_float2(split > 0 ? a : b, split > 1 ? a : b);
                 m23 = make_float2(split > 2 ? a : b, split > 3 ? a : b);
             }
-            e01 = __fmul2_rn(__fadd2_rn(d01, m01), make_float2(x.g.x, x.g.y));
-            e23 = __fmul2_rn(__fadd2_rn(d23, m23), make_float2(x.g.z, x.g.w));
+            if (EXTRA == kStacked) {
+                const float2 r2 = make_float2(x.cr, x.cr);
+                e01 = __fadd2_rn(__fadd2_rn(__fadd2_rn(d01, m01), r2), cc01);
+                e23 = __fadd2_rn(__fadd2_rn(__fadd2_rn(d23, m23), r2), cc23);
+                e01 = __fmul2_rn(e01, make_float2(x.g.x, x.g.y));
+                e23 = __fmul2_rn(e23, make_float2(x.g.z, x.g.w));
+            } else {
+                e01 = __fmul2_rn(__fadd2_rn(d01, m01), make_float2(x.g.x, x.g.y));
+                e23 = __fmul2_rn(__fadd2_rn(d23, m23), make_float2(x.g.z, x.g.w));
+            }
+            if (EXTRA == kMultiGain) {
+                // words of the higher stages (few pixels) are redone one by
+                // one: e = (value - pedestal) * inv_gain of their stage, no
+                // common mode, 0 past the last stage
+                const uint32_t hi = 0x10001u * (0xFFFFu & ~mg.vmask);
+                if ((x.rw.x | x.rw.y) & hi) {
+                    const size_t px = mod_base + (size_t)(r0 - 1 + rl) * p.cols + col;
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const uint32_t w = ((i < 2 ? x.rw.x : x.rw.y) >> (16 * (i & 1))) & 0xFFFFu;
+                        if (w >> mg.shift) {
+                            const float e = mg_energy(mg, p.frame_px, (uint16_t)w, px + i, 0.0f);
+                            if (i == 0) e01.x = e;
+                            if (i == 1) e01.y = e;
+                            if (i == 2) e23.x = e;
+                            if (i == 3) e23.y = e;
+                        }
+                    }
+                }
+            }
         };
         auto load = [&](int r) -> LeanRow {
             const uint32_t off = (uint32_t)r * p.cols + (uint32_t)col;
@@ -684,6 +733,7 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const uint16_t* 
                 x.rw = __ldg(reinterpret_cast<const uint2*>(fr + off));
             x.np = __ldg(reinterpret_cast<const float4*>(npm + off));
             x.g = __ldg(reinterpret_cast<const float4*>(gm + off));
+            x.cr = EXTRA == kStacked ? -__ldg(cmr + r) : 0.0f;
             return x;
         };
 
@@ -719,16 +769,22 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const uint16_t* 
                           : rows_here > (int)ty  ? (rows_here - 1 - (int)ty) / (int)TY + 1
                                                  : 0;
         uint32_t cmask = 0;  // bit i: own row i may hold a candidate
+        // (clamped below before the offset goes, so that the difference of an
+        // energy far below the histogram does not wrap)
+        auto bin_of = [&](float u) {
+            return __viaddmin_s32(max(__float_as_int(u), (int)kMagicBits), -(int)kMagicBits,
+                                  last_bin);
+        };
         auto own_row = [&](const LeanRow& x, int i) {
             const int rl = 1 + (int)ty + i * (int)TY;
             float2 e01, e23;
             correct(x, rl, e01, e23);
             const float2 u01 = __fadd2_rd(__ffma2_rn(e01, iw2, nl2), mg2);
             const float2 u23 = __fadd2_rd(__ffma2_rn(e23, iw2, nl2), mg2);
-            const int b0 = min(__viaddmax_s32(__float_as_int(u01.x), -(int)kMagicBits, 0), last_bin);
-            const int b1 = min(__viaddmax_s32(__float_as_int(u01.y), -(int)kMagicBits, 0), last_bin);
-            const int b2 = min(__viaddmax_s32(__float_as_int(u23.x), -(int)kMagicBits, 0), last_bin);
-            const int b3 = min(__viaddmax_s32(__float_as_int(u23.y), -(int)kMagicBits, 0), last_bin);
+            const int b0 = bin_of(u01.x);
+            const int b1 = bin_of(u01.y);
+            const int b2 = bin_of(u23.x);
+            const int b3 = bin_of(u23.y);
             atomicAdd(&hpix[b0], 1u);
             atomicAdd(&hpix[b1], 1u);
             atomicAdd(&hpix[b2], 1u);
@@ -880,12 +936,13 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const uint16_t* 
 // frames.  STAGE: the tile's raw rows come by one tensor copy (the frames as
 // [frame][period][group][8 words]) into shared memory; the next tile's copy
 // is issued once the rows are read and lands while the seeds are tested.
-// ONEUNIT: as in lean_tile.
-template <bool COLBANK, bool CORR, bool STAGE, bool ONEUNIT = false>
+// ONEUNIT, EXTRA: as in lean_tile.
+template <bool COLBANK, bool CORR, bool STAGE, bool ONEUNIT = false, int EXTRA = kPlain>
 __global__ void __launch_bounds__(kLeanThreads, 2)
     stencil_lean_kernel(ChainParams p, const uint16_t* __restrict__ raw, uint32_t frame_base,
                         CallOut out, LeanConfig lc, unsigned long long n_tiles,
-                        const __grid_constant__ CUtensorMap frames, uint32_t* __restrict__ err) {
+                        const __grid_constant__ CUtensorMap frames, uint32_t* __restrict__ err,
+                        MultiGain mg) {
     extern __shared__ __align__(128) float lean_smem[];
     __shared__ uint32_t list_n[2];
     __shared__ uint64_t stage_bar;
@@ -943,8 +1000,8 @@ __global__ void __launch_bounds__(kLeanThreads, 2)
     }
     uint32_t par = 0;
     for (unsigned long long t = first; t < n_tiles; t += step, walk.next(), par ^= 1u) {
-        const bool ok = lean_tile<COLBANK, CORR, STAGE, ONEUNIT>(
-            p, raw, frame_base, out, lc, sm, lane, walk.f, walk.m, walk.band, par, true, err, [&] {
+        const bool ok = lean_tile<COLBANK, CORR, STAGE, ONEUNIT, EXTRA>(
+            p, mg, raw, frame_base, out, lc, sm, lane, walk.f, walk.m, walk.band, par, true, err, [&] {
                 if (STAGE && t + step < n_tiles) {
                     fence_async_smem();  // order the generic reads of the stage before the copy
                     issue(t + step);
@@ -1138,8 +1195,8 @@ __global__ void __launch_bounds__(kBankThreads, 2)
                 if (!ok) atomicOr(err, 4u);
             }
             if (__syncthreads_or(!ok)) return;
-            lean_tile<true, false, false, false>(p, raw, frame_base, out, lc, ts, lane, f, m, band, par,
-                                          rowlane, err, [] {});
+            lean_tile<true, false, false, false, kPlain>(p, MultiGain{}, raw, frame_base, out, lc, ts,
+                                                         lane, f, m, band, par, rowlane, err, [] {});
             par ^= 1u;
             prev = 1;
         }
@@ -1225,7 +1282,6 @@ bool build_code_map(const ChainParams& p, const float* pedestal, std::vector<uin
     const size_t per_unit = (size_t)T * ne_box * 8;
     const uint16_t junk = (uint16_t)(bias + 4096);
     kmap->assign((size_t)p.units_per_frame * per_unit, junk);
-    const size_t tpx = (size_t)T * p.cols;  // words per period
     for (uint32_t u = 0; u < p.units_per_frame; u++) {
         uint32_t R0, c0;
         unit_pos(u, &R0, &c0);
@@ -1233,19 +1289,16 @@ bool build_code_map(const ChainParams& p, const float* pedestal, std::vector<uin
         for (uint32_t ph = 0; ph < T; ph++) {
             uint16_t* dst = kmap->data() + (size_t)u * per_unit + (size_t)ph * ne_box * 8;
             const uint32_t g_lo = (ph * p.cols + c0) / 8;
-            for (uint32_t pp = 0; pp < bp; pp++)
-                for (uint32_t k = 0; k < w8; k++)
-                    for (uint32_t l = 0; l < 8; l++) {
-                        const size_t ppx = 8 * ((size_t)g_lo + k) + l;  // word of the period
-                        if (ppx >= tpx) continue;
-                        const uint32_t rp = (uint32_t)(ppx / p.cols);
-                        const uint32_t col = (uint32_t)(ppx % p.cols);
-                        const size_t R = (size_t)(q_lo + pp) * T + rp;
-                        if (rp != ph || R < R0 || R >= (size_t)R0 + p.unit_rows || col < c0 ||
-                            col >= c0 + p.unit_cols)
-                            continue;
-                        dst[((size_t)pp * w8 + k) * 8 + l] = (uint16_t)(F[R * p.cols + col] + bias);
-                    }
+            // word w of a box row is column 8 g_lo + w - ph cols of the row
+            const long long first = 8ll * g_lo - (long long)ph * p.cols;
+            for (uint32_t pp = 0; pp < bp; pp++) {
+                const size_t R = (size_t)(q_lo + pp) * T + ph;
+                if (R < R0 || R >= (size_t)R0 + p.unit_rows) continue;
+                const int32_t* row = F.data() + R * p.cols;
+                uint16_t* line = dst + (size_t)pp * w8 * 8;
+                for (uint32_t col = c0; col < c0 + p.unit_cols; col++)
+                    line[(long long)col - first] = (uint16_t)(row[col] + bias);
+            }
         }
     }
     *out = CodeMap{nullptr, w8, (uint32_t)bias, (uint32_t)rcap, T, bp, ne_box, 2};
@@ -1341,14 +1394,14 @@ void set_stage_periods(LeanConfig& lc) {
 }
 bool staged(const LeanConfig& lc) { return lc.stage_t != 0 && lc.stage_bp <= 256; }
 
-LeanConfig make_lean_config(const ChainParams& p, uint32_t rb) {
+LeanConfig make_lean_config(const ChainParams& p, uint32_t rb, bool multigain) {
     LeanConfig lc{};
     lc.ok = false;
     // four-pixel chunks start 8-byte aligned in every frame and module, and a
     // chunk takes the common mode of at most two units
     if (p.cols % 4 || p.module_px % 4 || p.frame_px % 4 || p.unit_cols < 2) return lc;
     if (p.cols / 4 > kLeanThreads || p.cols > 65535) return lc;
-    if (cm_kind(p) == PD_CM_MEAN_STACKED || cm_after_gain(p)) return lc;
+    if (cm_after_gain(p)) return lc;
     lc.tx = p.cols / 4;
     lc.ty = std::max<uint32_t>(1, kLeanThreads / lc.tx);
     lc.pitch = p.cols + 8;
@@ -1393,7 +1446,9 @@ LeanConfig make_lean_config(const ChainParams& p, uint32_t rb) {
     // (measured 117.7 k against 122.1 k frames/s), so it stays off there.
     // (nor a CTA per SM: a band that fits two CTAs per SM unstaged keeps them)
     const size_t stage_limit = lean_smem_bytes(p, lc) <= kLeanSmemTwo ? kLeanSmemTwo : limit;
-    for (uint32_t t = 1; t <= 8 && lc.ok; t *= 2)
+    // (and the stacked mean and auto-ranging instances read raw unstaged)
+    const bool plain = cm_kind(p) != PD_CM_MEAN_STACKED && !multigain;
+    for (uint32_t t = 1; t <= 8 && lc.ok && plain; t *= 2)
         if ((t * p.cols) % 8 == 0) {
             if (t * p.cols / 8 <= 256 && (p.frame_px / p.cols) % t == 0 && p.frame_px % 8 == 0 &&
                 encode_fn() != nullptr) {
@@ -1418,6 +1473,12 @@ static int g_attr_dev_lean = -1;
 namespace {
 // the stencil instance for a common-mode layout: column banks, a per-row
 // table, or a per-row table whose chunks each lie in one unit
+template <bool CORR, int EXTRA>
+auto lean_pick_extra(bool colbank) {
+    return colbank ? stencil_lean_kernel<true, CORR, false, false, EXTRA>
+                   : stencil_lean_kernel<false, CORR, false, false, EXTRA>;
+}
+
 template <bool CORR, bool STAGE>
 auto lean_pick(bool colbank, bool oneunit) {
     return colbank   ? stencil_lean_kernel<true, CORR, STAGE, false>
@@ -1428,7 +1489,7 @@ auto lean_pick(bool colbank, bool oneunit) {
 
 cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& lc, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
-                                uint32_t* err, cudaStream_t stream) {
+                                uint32_t* err, cudaStream_t stream, const MultiGain* mg) {
     const unsigned long long n_tiles = (unsigned long long)n_frames * p.n_modules * lc.n_bands;
     if (n_tiles == 0) return cudaSuccess;
     int dev = 0;
@@ -1441,7 +1502,12 @@ cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& lc, cons
                        stencil_lean_kernel<false, false, false, true>,
                        stencil_lean_kernel<false, true, false, true>,
                        stencil_lean_kernel<false, false, true, true>,
-                       stencil_lean_kernel<false, true, true, true>}) {
+                       stencil_lean_kernel<false, true, true, true>,
+                       lean_pick_extra<false, kStacked>(true), lean_pick_extra<true, kStacked>(true),
+                       lean_pick_extra<false, kStacked>(false), lean_pick_extra<true, kStacked>(false),
+                       lean_pick_extra<false, kMultiGain>(true), lean_pick_extra<true, kMultiGain>(true),
+                       lean_pick_extra<false, kMultiGain>(false),
+                       lean_pick_extra<true, kMultiGain>(false)}) {
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)kLeanSmemMax);
             if (e == cudaSuccess)
@@ -1481,7 +1547,14 @@ cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& lc, cons
                            : lean_pick<false, true>(lc.colbank, one))
                    : (corr ? lean_pick<true, false>(lc.colbank, one)
                            : lean_pick<false, false>(lc.colbank, one));
-    k<<<(unsigned)grid, threads, smem, stream>>>(p, raw, frame_base, out, lc, n_tiles, map, err);
+    if (mg)
+        k = corr ? lean_pick_extra<true, kMultiGain>(lc.colbank)
+                 : lean_pick_extra<false, kMultiGain>(lc.colbank);
+    else if (cm_kind(p) == PD_CM_MEAN_STACKED)
+        k = corr ? lean_pick_extra<true, kStacked>(lc.colbank)
+                 : lean_pick_extra<false, kStacked>(lc.colbank);
+    k<<<(unsigned)grid, threads, smem, stream>>>(p, raw, frame_base, out, lc, n_tiles, map, err,
+                                                 mg ? *mg : MultiGain{});
     return cudaGetLastError();
 }
 

@@ -74,13 +74,15 @@ struct LeanConfig {
     bool ok;
 };
 
-LeanConfig make_lean_config(const ChainParams& p, uint32_t rb = 0);
+// multigain: the words are auto-ranging ones.
+LeanConfig make_lean_config(const ChainParams& p, uint32_t rb = 0, bool multigain = false);
 size_t lean_smem_bytes(const ChainParams& p, const LeanConfig& lc);
 // raw: 16-byte aligned.  err: context error word (bit 1: a bounded wait
-// for a staged copy gave up).
+// for a staged copy gave up).  mg: auto-ranging words, or NULL.
 cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& lc, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
-                                uint32_t* err, cudaStream_t stream);
+                                uint32_t* err, cudaStream_t stream,
+                                const MultiGain* mg = nullptr);
 
 // The lean pair as one persistent launch over a work queue (bank items of
 // frames [sK, sK + K) then the stencil tiles of the K frames before them, K
