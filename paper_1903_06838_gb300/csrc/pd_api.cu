@@ -57,6 +57,9 @@ struct pd_ctx {
     bool use_bank = false, use_lean = false;
     pd::CodeMap cmap{};
     uint4* d_kmap = nullptr;
+    bool use_row_codes = false;  // one-row units by 16-bit codes (pd_rows.cu)
+    pd::RowCodes row_codes{};
+    uint16_t* d_row_kmap = nullptr;
     pd::LeanConfig lean_cfg{};
     uint32_t kernels = 1;       // 1: the lean pair where available; 2: the earlier pair;
                                 // 3: the lean pair as one work-queue launch
@@ -221,6 +224,7 @@ void free_ctx(pd_ctx* c) {
     cudaFree(c->d_mg_ped);
     cudaFree(c->d_mg_ig);
     cudaFree(c->d_kmap);
+    cudaFree(c->d_row_kmap);
     cudaFree(c->d_qsync);
     cudaFree(c->d_err);
     cudaFree(c->d_stage[0]);
@@ -279,6 +283,8 @@ cudaError_t launch_cm(const pd_ctx* c, const uint16_t* fr, uint32_t nf, float* c
         cmap.wait_polls = c->wait_polls;
         return pd::launch_cm_bank(c->params, c->cm_cfg, cmap, fr, nf, cm, c->d_err, s);
     }
+    if (c->use_row_codes && c->kernels == 1)
+        return pd::launch_row_codes(c->params, c->row_codes, fr, nf, cm, s);
     if (c->multigain)
         return c->use_cm_big ? pd::launch_cm_big(c->params, c->cm_cfg, fr, nf, cm, s,
                                                  ~c->mg.vmask & 0xFFFFu)
@@ -657,28 +663,44 @@ int create_impl(const pd_geometry* geometry, uint32_t n_gains, uint32_t gain_shi
         c->lean_cfg = pd::make_lean_config(p, 0, c->multigain);
         c->use_lean = c->lean_cfg.ok;
         std::vector<uint16_t> km;
-        pd::CodeMap cmap{};
+        auto upload = [&](void* dst) -> int {
+            if (cudaMalloc((void**)dst, km.size() * 2) != cudaSuccess)
+                return fail(PD_ENOMEM, "device allocation failed in pd_create");
+            const cudaError_t ce =
+                cudaMemcpy(*(void**)dst, km.data(), km.size() * 2, cudaMemcpyHostToDevice);
+            return ce == cudaSuccess ? PD_OK : fail_cuda(ce, "pd_create upload");
+        };
         // Auto-ranging words outside stage 0 are at least 2^gain_shift.  Where
         // the raw cap lies no higher, they take the code of a word at the cap,
         // the spare bin of d >= cut, and the whole-unit selection's d (stage
-        // 0's pedestal) is past the cut too: the bank median reads them as it
-        // reads single-gain words (64 frames of 32 x 185 x 388: 257 us with the
-        // floating-point bank median, 222 us).
+        // 0's pedestal) is past the cut too: the coded medians read them as
+        // they read single-gain words (64 frames of 32 x 185 x 388: 257 us
+        // with the floating-point bank median, 222 us).
+        auto readable = [&](uint32_t rcap) { return !n_gains || rcap <= (1u << gain_shift); };
+        pd::CodeMap cmap{};
+        pd::RowCodes rows{};
         if (c->use_cm_big && pd::build_code_map(p, pedestal_host, &km, &cmap) &&
-            pd::cm_bank_supported(p, cmap) && (!n_gains || cmap.rcap <= (1u << gain_shift))) {
-            if ((e = cudaMalloc(&c->d_kmap, km.size() * 2)) != cudaSuccess) {
+            pd::cm_bank_supported(p, cmap) && readable(cmap.rcap)) {
+            rc = upload(&c->d_kmap);
+            if (rc) {
                 free_ctx(c);
-                return fail(PD_ENOMEM, "device allocation failed in pd_create");
-            }
-            if ((e = cudaMemcpy(c->d_kmap, km.data(), km.size() * 2, cudaMemcpyHostToDevice))) {
-                free_ctx(c);
-                return fail_cuda(e, "pd_create upload");
+                return rc;
             }
             cmap.kmap = c->d_kmap;
             c->cmap = cmap;
             c->use_bank = true;
             c->use_queue =
                 c->use_lean && !c->multigain && pd::queue_supported(p, cmap, c->lean_cfg);
+        } else if (g.cm_mode == PD_CM_MEDIAN && !c->use_cm_big &&
+                   pd::build_row_codes(p, pedestal_host, &km, &rows) && readable(rows.rcap)) {
+            rc = upload(&c->d_row_kmap);
+            if (rc) {
+                free_ctx(c);
+                return rc;
+            }
+            rows.kmap = c->d_row_kmap;
+            c->row_codes = rows;
+            c->use_row_codes = true;
         }
     }
     pd::noalloc_prepare(c->device);
@@ -924,7 +946,7 @@ int pd_get_tuning(const pd_ctx* c, pd_tuning* t) {
     t->band_rows = lean ? c->lean_cfg.rb : c->use_band ? c->band_cfg.rb : 0;
     t->overlap = c->overlap;
     t->two_pass = c->use_fused && !c->matched ? c->two_pass : 1;
-    t->kernels = c->use_lean || c->use_bank ? (c->kernels == 3 && !c->use_queue ? 1u : c->kernels)
+    t->kernels = c->use_lean || c->use_bank || c->use_row_codes ? (c->kernels == 3 && !c->use_queue ? 1u : c->kernels)
                                             : 2;
     return PD_OK;
 }
@@ -1366,7 +1388,7 @@ int pd_autotune(pd_ctx* c, const uint16_t* frames_dev, uint32_t n_frames, pd_tun
         if (c->use_fused && !c->matched)
             cands.push_back(pd_tuning{orig.chunk_frames, orig.band_rows, 1, 0, orig.kernels});
         std::vector<uint32_t> kopts = {orig.kernels};
-        if ((c->use_lean || c->use_bank) && !c->matched) kopts = {1u, 2u};
+        if ((c->use_lean || c->use_bank || c->use_row_codes) && !c->matched) kopts = {1u, 2u};
         // the work-queue launch: one launch per call, so chunking, band
         // height and overlap are not varied
         if (c->use_queue && !c->matched) cands.push_back(pd_tuning{orig.chunk_frames, 0, 1, 1, 3});

@@ -1224,44 +1224,52 @@ long long floor_sum(double a, double b) {
 
 }  // namespace
 
+bool code_base(const ChainParams& p, const float* pedestal, int n_codes, CodeBase* out) {
+    if (!(p.cm_cut > -1e6f && p.cm_cut < 1e6f)) return false;
+    const double cut = p.cm_cut;
+    const double lo = cut - n_codes / 8.0;
+    const size_t fpx = p.frame_px;
+    long long fmin = 0, fmax = 0;
+    float least = INFINITY;  // smallest nonzero |pedestal|
+    out->F.resize(fpx);
+    for (size_t i = 0; i < fpx; i++) {
+        const float ped = pedestal[i];
+        if (!std::isfinite(ped)) return false;
+        if (ped != 0.0f) least = std::min(least, std::fabs(ped));
+        const long long fv = floor_sum(-8.0 * (double)ped, -8.0 * lo);
+        if (fv < -(1LL << 30) || fv > (1LL << 30)) return false;
+        out->F[i] = (int32_t)fv;
+        fmin = i ? std::min(fmin, fv) : fv;
+        fmax = i ? std::max(fmax, fv) : fv;
+    }
+    if (std::isfinite(least)) {
+        // d = x - ped is exact in binary32 while |d| < 2^24 ulp-units of ped
+        int ex = 0;
+        std::frexp((double)least, &ex);  // least in [2^(ex-1), 2^ex)
+        const int q = std::max(ex - 24, -149);
+        const double D = std::max(std::fabs(lo), std::fabs(cut));
+        if (!(D < std::ldexp(1.0, 24 + q))) return false;
+    }
+    // raw words at or above ceil((n_codes - F) / 8) are in the spare bin
+    const long long need = n_codes - fmin;
+    out->rcap = need <= 0 ? 0 : (need + 7) / 8;
+    out->bias = fmin < 0 ? -fmin : 0;
+    const long long kmax = std::max(fmax + out->bias, out->bias + n_codes);
+    return out->rcap <= 65535 && 8 * out->rcap + kmax <= 65535;
+}
+
 bool build_code_map(const ChainParams& p, const float* pedestal, std::vector<uint16_t>* kmap,
                     CodeMap* out) {
     if (p.frame_px % 8) return false;
-    if (!(p.cm_cut > -1e6f && p.cm_cut < 1e6f)) return false;
     // periods of t rows whose length is a multiple of 8 words tile the frame
     uint32_t gcd = 8;
     while (p.cols % gcd) gcd >>= 1;
     const uint32_t T = 8 / gcd;
     if (((size_t)p.n_modules * p.rows) % T) return false;
-    const double cut = p.cm_cut;
-    const double lo = cut - 512.0;
-    const double D = std::max(std::fabs(lo), std::fabs(cut));
-    const size_t fpx = p.frame_px;
-    long long fmin = 0, fmax = 0, rcap = 0;
-    std::vector<int32_t> F(fpx);
-    for (size_t i = 0; i < fpx; i++) {
-        const float ped = pedestal[i];
-        if (!std::isfinite(ped)) return false;
-        if (ped != 0.0f) {
-            // d = x - ped is exact in binary32 while |d| < 2^24 ulp-units of ped
-            int ex = 0;
-            std::frexp((double)ped, &ex);  // |ped| in [2^(ex-1), 2^ex)
-            const int q = std::max(ex - 24, -149);
-            if (!(D < std::ldexp(1.0, 24 + q))) return false;
-        }
-        const long long fv = floor_sum(-8.0 * (double)ped, -8.0 * lo);
-        if (fv < -(1LL << 30) || fv > (1LL << 30)) return false;
-        F[i] = (int32_t)fv;
-        // raw words at or above ceil((4096 - F) / 8) are in the spare bin
-        const long long need = 4096 - fv;
-        const long long rc = need <= 0 ? 0 : (need + 7) / 8;
-        fmin = i ? std::min(fmin, fv) : fv;
-        fmax = i ? std::max(fmax, fv) : fv;
-        rcap = i ? std::max(rcap, rc) : rc;
-    }
-    const long long bias = fmin < 0 ? -fmin : 0;
-    const long long kmax = std::max(fmax + bias, bias + 4096);
-    if (rcap > 65535 || 8 * rcap + kmax > 65535) return false;
+    CodeBase cb;
+    if (!code_base(p, pedestal, (int)kCmBins, &cb)) return false;
+    const std::vector<int32_t>& F = cb.F;
+    const long long bias = cb.bias, rcap = cb.rcap;
     // box of a unit's rows of one phase: periods q_lo .. q_hi, groups
     // g_lo(phase) .. g_hi(phase) of a period
     auto unit_pos = [&](uint32_t u, uint32_t* R0, uint32_t* c0) {

@@ -40,6 +40,28 @@ struct CodeMap {
     uint32_t wait_polls;   // polls of a copy's mbarrier before giving up (0: default)
 };
 
+// Host side of the integer codes of a window of n_codes / 8 ADU below the cut
+// (lo = cut - n_codes / 8): F of every pixel, the bias that makes the offsets
+// non-negative and the raw cap; false when the codes are not exact or do not
+// fit 16-bit lanes.
+struct CodeBase {
+    std::vector<int32_t> F;
+    long long bias, rcap;
+};
+bool code_base(const ChainParams& p, const float* pedestal, int n_codes, CodeBase* out);
+
+// One-row units by 16-bit codes (pd_rows.cu): the offsets K' in frame order,
+// codes from `first` (the window's lower edge and everything below) to
+// `spare` (d >= cut).
+struct RowCodes {
+    const uint16_t* kmap;  // [frame_px]
+    uint32_t rcap, first, spare;
+};
+bool build_row_codes(const ChainParams& p, const float* pedestal, std::vector<uint16_t>* kmap,
+                     RowCodes* out);
+cudaError_t launch_row_codes(const ChainParams& p, const RowCodes& rc, const uint16_t* raw,
+                             uint32_t n_frames, float* cm, cudaStream_t stream);
+
 // Host side: the map of a geometry and pedestal (out->kmap left null), or
 // false when the integer codes are not exact, do not fit 16-bit lanes, or the
 // boxes exceed the tensor copy's limits (the context then keeps the
