@@ -153,8 +153,9 @@ struct pd_net {
     uint8_t* tc_img = nullptr;
     uint16_t* tc_h2 = nullptr;
     int* tc_err = nullptr;
-    // training: bf16 weight fragments, bf16 h2 and dz3 rows
+    // training: bf16 weight fragments, bf16 h2 and dz3 rows, gradient sums
     uint4* tr_img = nullptr;
+    float* tr_slices = nullptr;
     uint16_t *tr_h2 = nullptr, *tr_dz3 = nullptr;
 };
 
@@ -169,6 +170,7 @@ void free_net(pd_net* n) {
     cudaFree(n->tr_img);
     cudaFree(n->tr_h2);
     cudaFree(n->tr_dz3);
+    cudaFree(n->tr_slices);
     delete n;
 }
 
@@ -195,6 +197,8 @@ int pd_net_create(uint32_t max_batch, uint64_t seed, pd_net** out) {
         cudaMalloc(&n->tr_img, pd::nettrain::image_bytes()) != cudaSuccess ||
         cudaMalloc(&n->tr_h2, pd::nettrain::h2_bytes(max_batch)) != cudaSuccess ||
         cudaMalloc(&n->tr_dz3, pd::nettrain::dz3_bytes(max_batch)) != cudaSuccess ||
+        cudaMalloc(&n->tr_slices, pd::nettrain::slice_bytes(max_batch, pd::device_sm_count())) !=
+            cudaSuccess ||
         cudaMemset(n->tc_err, 0, sizeof(int)) != cudaSuccess) {
         free_net(n);
         return net_fail(PD_ENOMEM, "pd_net_create: device allocation failed");
@@ -274,7 +278,8 @@ int pd_net_gradients(pd_net* n, const float* patches, const uint8_t* counts, con
     float* g = grads_dev && (uintptr_t)grads_dev % 8 == 0 ? grads_dev : n->gw;
     cudaError_t e = pd::nettrain::gradients(n->w, patches, counts, targets, mask, count,
                                             std::max(1.0f, n_reg), lambda, n->tr_img, n->tr_h2,
-                                            n->tr_dz3, g, loss_dev, pd::device_sm_count(), s);
+                                            n->tr_dz3, n->tr_slices, g, loss_dev,
+                                            pd::device_sm_count(), s);
     if (!e && grads_dev && g != grads_dev)
         e = cudaMemcpyAsync(grads_dev, g, NPARAM * 4, cudaMemcpyDeviceToDevice, s);
     return e == cudaSuccess ? PD_OK : net_cuda(e, "pd_net_gradients");

@@ -12,8 +12,14 @@
 //                  16-deep step are one 16-byte load), and the gradients zero
 //   step_kernel    conv1, conv2, FC3, heads, loss, and back to conv1; every
 //                  weight gradient but W3's is summed in registers over the
-//                  CTA's tiles and added to the result once
-//   wgrad3_kernel  W3's gradient, dz3^T h2 over slices of 128 hits
+//                  CTA's tiles and written to the CTA's slice once
+//   finish_kernel  the sum of the slices, and W3's gradient, dz3^T h2 over
+//                  128 hits a block
+//
+// (256 CTAs adding their 9,568 sums to the result atomically took 13 of the
+// step kernel's 35 us.)  Each launch starts while the one before ends
+// (programmatic dependent launch): step_kernel clears its shared memory
+// during prep_kernel.
 //
 // Eight hits are 200 (hit, position) rows, thirteen 16-row tiles, and one
 // n-tile of FC3 and its transpose, where the weights are the 16-row operand;
@@ -42,6 +48,9 @@ constexpr int NPOS = 25, C1 = 32, C2 = 32, NH = 64, NOUT = 7, K3 = NPOS * C2;
 constexpr int OW1 = 0, OB1 = OW1 + C1 * 9, OW2 = OB1 + C1, OB2 = OW2 + C2 * 9 * C1,
               OW3 = OB2 + C2, OB3 = OW3 + NH * K3, OW4 = OB3 + NH, OB4 = OW4 + NOUT * NH,
               NPARAM = OB4 + NOUT;
+// a CTA's slice of sums: the parameters before W3, those after it, the loss
+constexpr int SL_TAIL = OW3, SL_LOSS = OW3 + NPARAM - OB3, SLICE = SL_LOSS + 1;
+static_assert(SLICE % 4 == 0, "slices are read four floats at a time");
 
 // fragment images (16-byte units: one lane's share of a 16-deep step)
 constexpr int I_W3 = 0;                  // FC3, rows = outputs: [4][50][32]
@@ -120,6 +129,12 @@ __device__ __forceinline__ void ldsm2t(uint32_t addr, uint32_t (&r)[2]) {
                  : "=r"(r[0]), "=r"(r[1])
                  : "r"(addr));
 }
+// the kernel before this one in the stream is complete, its writes visible
+__device__ __forceinline__ void wait_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// the next kernel in the stream may start (and wait for this one's end)
+__device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;"); }
 // two neighbouring floats of the result (8-byte aligned), added atomically
 __device__ __forceinline__ void add2(float* dst, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dst), "f"(a), "f"(b) : "memory");
@@ -134,7 +149,8 @@ __host__ __device__ constexpr int tap_off(int k) { return (k / 3 - 1) * 7 + k % 
 // elements (g, 2t..), (g + 8, 2t..), (g, 2t + 8..), (g + 8, 2t + 8..), of B
 // (k = 2t.., n = g), (k = 2t + 8.., n = g); a B image unit holds two n-tiles.
 __global__ void prep_kernel(const float* __restrict__ w, uint4* __restrict__ img,
-                            float* __restrict__ grads) {
+                            float* __restrict__ gw3) {
+    start_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < I_ALL) {
         const int lane = i & 31, g = lane >> 2, t = lane & 3;
@@ -168,7 +184,7 @@ __global__ void prep_kernel(const float* __restrict__ w, uint4* __restrict__ img
         }
         img[i] = make_uint4(q[0], q[1], q[2], q[3]);
     }
-    for (int k = i; k < NPARAM; k += gridDim.x * blockDim.x) grads[k] = 0.0f;
+    for (int k = i; k < NH * K3; k += gridDim.x * blockDim.x) gw3[k] = 0.0f;
 }
 
 // acc[m][n] = rows x weights of a 3x3 convolution over the padded grids at
@@ -214,7 +230,7 @@ __global__ void __launch_bounds__(THREADS, 2)
                 const float* __restrict__ x, const uint8_t* __restrict__ counts,
                 const float* __restrict__ tgt, const uint8_t* __restrict__ mask, int n, float nreg,
                 float lam, uint16_t* __restrict__ h2_out, uint16_t* __restrict__ dz3_out,
-                float* __restrict__ gw, float* __restrict__ loss) {
+                float* __restrict__ slices) {
     extern __shared__ __align__(128) uint8_t sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, tq = lane & 3;
@@ -245,6 +261,7 @@ __global__ void __launch_bounds__(THREADS, 2)
 #pragma unroll
     for (int c = 0; c < 8; c++) gb1[c] = 0.0f;
 
+    wait_previous();  // the weight images
     const int n_tiles = (n + HB - 1) / HB;
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         const int hit0 = t * HB, nh = min(HB, n - hit0);
@@ -532,56 +549,112 @@ __global__ void __launch_bounds__(THREADS, 2)
         }
     }
 
-    // the CTA's sums into the result
+    // the CTA's sums into its slice: W2's straight from registers, the others
+    // summed over the warps in shared memory first
+    start_next();
+    float* slice = slices + (size_t)blockIdx.x * SLICE;
+    constexpr int F_B1 = 288, F_B2 = F_B1 + C1, F_TAIL = F_B2 + C2, F_ALL = F_TAIL + SLICE - SL_TAIL;
+    static_assert(F_ALL <= 2 * NH * HB, "the small sums fit the FC3 halves");
+    for (int i = tid; i < F_ALL; i += THREADS) s_red[i] = 0.0f;
     {
         const int co = (warp & 1) * 16 + g, ci = (warp >> 1) * 8 + 2 * tq;
-        float* d = gw + OW2 + co * (9 * C1) + ci;
+        float* d = slice + OW2 + co * (9 * C1) + ci;
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            add2(d + k * C1, gw2[k][0], gw2[k][1]);
-            add2(d + 8 * 9 * C1 + k * C1, gw2[k][2], gw2[k][3]);
+            *reinterpret_cast<float2*>(d + k * C1) = make_float2(gw2[k][0], gw2[k][1]);
+            *reinterpret_cast<float2*>(d + 8 * 9 * C1 + k * C1) = make_float2(gw2[k][2], gw2[k][3]);
         }
     }
+    __syncthreads();
     {
         const int co = (warp & 1) * 16 + g, k = ((warp >> 1) & 1) * 8 + 2 * tq;
 #pragma unroll
         for (int c = 0; c < 4; c++)
-            if (k + (c & 1) < 9) atomicAdd(gw + OW1 + (co + 8 * (c >> 1)) * 9 + k + (c & 1), gw1[c]);
+            if (k + (c & 1) < 9)
+                atomicAdd(s_red + (co + 8 * (c >> 1)) * 9 + k + (c & 1), gw1[c]);
     }
 #pragma unroll
     for (int c = 0; c < 8; c++) {
         float v = gb1[c];
 #pragma unroll
         for (int b = 4; b < 32; b <<= 1) v += __shfl_xor_sync(0xffffffffu, v, b);
-        if (g == 0) atomicAdd(gw + OB1 + (c >> 1) * 8 + 2 * tq + (c & 1), v);
+        if (g == 0) atomicAdd(s_red + F_B1 + (c >> 1) * 8 + 2 * tq + (c & 1), v);
     }
 #pragma unroll
     for (int c = 0; c < 2; c++) {
         float v = gb2[c];
 #pragma unroll
         for (int b = 1; b < 4; b <<= 1) v += __shfl_xor_sync(0xffffffffu, v, b);
-        if (tq == 0) atomicAdd(gw + OB2 + (warp & 1) * 16 + g + 8 * c, v);
-        atomicAdd(gw + OB3 + lane + 32 * c, gb3[c]);
+        if (tq == 0) atomicAdd(s_red + F_B2 + (warp & 1) * 16 + g + 8 * c, v);
+        atomicAdd(s_red + F_TAIL + lane + 32 * c, gb3[c]);
         const int q = tid + c * THREADS;
-        if (q < NOUT * NH) atomicAdd(gw + OW4 + q, gw4[c]);
+        if (q < NOUT * NH) s_red[F_TAIL + OW4 - OB3 + q] = gw4[c];
     }
-    if (tid < NOUT) atomicAdd(gw + OB4 + tid, gb4);
-    if (lane == 0 && loss) atomicAdd(loss, l_sum);
+    if (tid < NOUT) s_red[F_TAIL + OB4 - OB3 + tid] = gb4;
+    if (lane == 0) atomicAdd(s_red + F_TAIL + SL_LOSS - SL_TAIL, l_sum);
+    __syncthreads();
+    for (int i = tid; i < F_ALL; i += THREADS) {
+        const int at = i < F_B1 ? OW1 + i : i < F_B2 ? OB1 + i - F_B1
+                     : i < F_TAIL ? OB2 + i - F_B2 : SL_TAIL + i - F_TAIL;
+        slice[at] = s_red[i];
+    }
 }
 
 // ---------------------------------------------------------------------------
-// gw3[64][800] += dz3^T h2 over the block's 128 hits, 80 columns: both
-// operands are read transposed from their rows in shared memory.
+// The first SUM_BLOCKS blocks sum 128 places of the slices each (a warp every
+// eighth slice); the others add dz3^T h2 over 128 hits to 80 columns of
+// gw3[64][800], both operands read transposed from their rows in shared memory.
 constexpr int W3_HITS = 128, W3_COLS = 80, W3_HP = 176;
+constexpr int SUM_BLOCKS = (SLICE / 4 + 31) / 32;
+
+__device__ __forceinline__ void sum_slices(const float* __restrict__ slices, int n_slices,
+                                           float* __restrict__ grads, float* __restrict__ loss,
+                                           float4 (*part)[32]) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q = blockIdx.x * 32 + lane;
+    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (q < SLICE / 4)
+#pragma unroll 8
+        for (int i = warp; i < n_slices; i += THREADS / 32) {
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(slices + (size_t)i * SLICE) + q);
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
+        }
+    part[warp][lane] = a;
+    __syncthreads();
+    if (threadIdx.x < 128) {
+        const float* f = reinterpret_cast<const float*>(part) + threadIdx.x;
+        float v = 0.0f;
+#pragma unroll
+        for (int k = 0; k < THREADS / 32; k++) v += f[k * 128];
+        const int at = blockIdx.x * 128 + threadIdx.x;
+        if (at < SL_TAIL)
+            grads[at] = v;
+        else if (at < SL_LOSS)
+            grads[OB3 + at - SL_TAIL] = v;
+        else if (at == SL_LOSS && loss)
+            atomicAdd(loss, v);
+    }
+}
 
 __global__ void __launch_bounds__(THREADS)
-    wgrad3_kernel(const uint16_t* __restrict__ dz3, const uint16_t* __restrict__ h2, int n,
-                  float* __restrict__ gw3) {
+    finish_kernel(const float* __restrict__ slices, int n_slices, const uint16_t* __restrict__ dz3,
+                  const uint16_t* __restrict__ h2, int n, float* __restrict__ grads,
+                  float* __restrict__ loss) {
     __shared__ __align__(128) uint8_t sd[W3_HITS * DP];
     __shared__ __align__(128) uint8_t sh[W3_HITS * W3_HP];
+    wait_previous();
+    if (blockIdx.x < SUM_BLOCKS) {
+        sum_slices(slices, n_slices, grads, loss, reinterpret_cast<float4 (*)[32]>(sd));
+        return;
+    }
+    const int block = blockIdx.x - SUM_BLOCKS;
+    float* gw3 = grads + OW3;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, tq = lane & 3;
-    const int col0 = blockIdx.x * W3_COLS, hit0 = blockIdx.y * W3_HITS;
+    const int col0 = block % (K3 / W3_COLS) * W3_COLS, hit0 = block / (K3 / W3_COLS) * W3_HITS;
     const int nh = min(W3_HITS, n - hit0);
     const uint32_t sda = (uint32_t)__cvta_generic_to_shared(sd);
     const uint32_t sha = (uint32_t)__cvta_generic_to_shared(sh);
@@ -637,11 +710,15 @@ __global__ void __launch_bounds__(THREADS)
 size_t image_bytes() { return (size_t)I_ALL * sizeof(uint4); }
 size_t h2_bytes(uint32_t max_batch) { return (size_t)max_batch * K3 * 2; }
 size_t dz3_bytes(uint32_t max_batch) { return (size_t)max_batch * NH * 2; }
+static uint32_t max_slices(int sms) { return 2u * (uint32_t)sms; }  // the persistent CTAs
+size_t slice_bytes(uint32_t max_batch, int sms) {
+    return (size_t)std::min((max_batch - 1) / HB + 1, max_slices(sms)) * SLICE * sizeof(float);
+}
 
 cudaError_t gradients(const float* w, const float* x, const uint8_t* counts, const float* targets,
                       const uint8_t* mask, uint32_t n, float n_reg, float lambda, uint4* img,
-                      uint16_t* h2, uint16_t* dz3, float* grads, float* loss, int sms,
-                      cudaStream_t s) {
+                      uint16_t* h2, uint16_t* dz3, float* slices, float* grads,
+                      float* loss, int sms, cudaStream_t s) {
     static int attr_dev = -1;  // the shared-memory opt-in, once per device
     int dev = 0;
     cudaGetDevice(&dev);
@@ -651,13 +728,27 @@ cudaError_t gradients(const float* w, const float* x, const uint8_t* counts, con
         if (e != cudaSuccess) return e;
         attr_dev = dev;
     }
-    prep_kernel<<<(I_ALL + 255) / 256, 256, 0, s>>>(w, img, grads);
-    const uint32_t tiles = (n + HB - 1) / HB;
-    step_kernel<<<std::min<uint32_t>(tiles, 2u * (uint32_t)sms), THREADS, S_BYTES, s>>>(
-        w, img, x, counts, targets, mask, (int)n, n_reg, lambda, h2, dz3, grads, loss);
-    wgrad3_kernel<<<dim3(K3 / W3_COLS, (n + W3_HITS - 1) / W3_HITS), THREADS, 0, s>>>(
-        dz3, h2, (int)n, grads + OW3);
-    return cudaGetLastError();
+    prep_kernel<<<(I_ALL + 255) / 256, 256, 0, s>>>(w, img, grads + OW3);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(THREADS);
+    cfg.stream = s;
+    cfg.attrs = &early;
+    cfg.numAttrs = 1;
+    const uint32_t grid = std::min((n - 1) / HB + 1, max_slices(sms));
+    cfg.gridDim = dim3(grid);
+    cfg.dynamicSmemBytes = S_BYTES;
+    e = cudaLaunchKernelEx(&cfg, step_kernel, w, (const uint4*)img, x, counts, targets, mask, (int)n,
+                           n_reg, lambda, h2, dz3, slices);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3(SUM_BLOCKS + K3 / W3_COLS * ((n + W3_HITS - 1) / W3_HITS));
+    cfg.dynamicSmemBytes = 0;
+    return cudaLaunchKernelEx(&cfg, finish_kernel, (const float*)slices, (int)grid,
+                              (const uint16_t*)dz3, (const uint16_t*)h2, (int)n, grads, loss);
 }
 
 }  // namespace nettrain
