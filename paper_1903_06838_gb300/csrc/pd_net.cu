@@ -73,41 +73,74 @@ __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ gr,
 // module): e recomputed exactly as the chain does, with the call's common
 // mode of frame - frame_base (unit term, and for the stacked mean the module
 // row and column terms).
+//
+// A warp takes kGatherHits hits, a lane per patch pixel.  With one hit a warp
+// the five integer divisions of its place were most of the instructions and
+// the kernel waited for one hit's loads at a time; now lane j splits hit j's
+// pixel and the others read it from there, units are found by multiplication,
+// and the loads of four hits are in flight.  300 thousand hits of 704 x 768
+// frames: 63 -> 32 us.
+constexpr int kGatherHits = 8;
+
+struct GatherDiv {  // ceil(2^32 / d) of the unit sizes, 0 for 1
+    uint32_t unit_rows, unit_cols;
+};
+// v / d for v < 2^16, d <= 2^16: with q = ceil(2^32 / d), v (q d - 2^32) < 2^32
+__device__ __forceinline__ uint32_t div16(uint32_t v, uint32_t q) {
+    return q ? __umulhi(v, q) : v;
+}
+
 template <bool MG>
-__global__ void gather_kernel(pd::ChainParams p, const uint16_t* __restrict__ raw,
-                              uint32_t frame_base, const float* __restrict__ cm,
-                              const pd_hit* __restrict__ hits, uint32_t n,
-                              float* __restrict__ patches, pd::MultiGain mg) {
-    const uint32_t h = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+__global__ void __launch_bounds__(256)
+    gather_kernel(pd::ChainParams p, const uint16_t* __restrict__ raw, uint32_t frame_base,
+                  const float* __restrict__ cm, const pd_hit* __restrict__ hits, uint32_t n,
+                  float* __restrict__ patches, pd::MultiGain mg, GatherDiv dv) {
+    const uint32_t h0 = (blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32) * kGatherHits;
     const int lane = threadIdx.x & 31;
-    if (h >= n || lane >= NPOS) return;
-    const pd_hit hit = hits[h];
-    const uint32_t f = hit.frame - frame_base;
-    const uint32_t m = hit.pixel / p.module_px, within = hit.pixel % p.module_px;
-    const int r = (int)(within / p.cols) + lane / 5 - 2, c = (int)(within % p.cols) + lane % 5 - 2;
-    float v = 0.0f;
-    if (r >= 0 && r < (int)p.rows && c >= 0 && c < (int)p.cols) {
-        const size_t g = (size_t)m * p.module_px + (size_t)r * p.cols + c;
-        const uint32_t unit = m * p.units_per_module +
-                              ((uint32_t)r / p.unit_rows) * p.units_per_row + (uint32_t)c / p.unit_cols;
-        const float* cmf = cm + (size_t)f * cm_per_frame(p);
-        float e;
-        if (MG) {
-            e = pd::mg_energy(mg, p.frame_px, raw[(size_t)f * p.frame_px + g], g, cmf[unit]);
-        } else {
-            const float d =
-                __fsub_rn(__uint2float_rn(raw[(size_t)f * p.frame_px + g]), p.ped[g]);
-            if (cm_kind(p) == PD_CM_MEAN_STACKED)
-                e = pd::energy<true>(cm_after_gain(p), d, p.inv_gain[g], cmf[unit],
-                                     cmf[p.units_per_frame + (size_t)m * p.rows + r],
-                                     cmf[p.units_per_frame + (size_t)p.n_modules * p.rows +
-                                         (size_t)m * p.cols + c]);
-            else
-                e = pd::energy<false>(cm_after_gain(p), d, p.inv_gain[g], cmf[unit], 0.0f, 0.0f);
+    if (h0 >= n) return;
+    const pd_hit* own = hits + min(h0 + (uint32_t)lane % kGatherHits, n - 1);
+    const uint32_t own_px = own->pixel, own_f = own->frame - frame_base;
+    const uint32_t own_m = own_px / p.module_px, within = own_px - own_m * p.module_px;
+    const uint32_t own_r = within / p.cols;
+    const uint32_t own_rc = own_r << 16 | (within - own_r * p.cols);
+    const int dy = lane / 5 - 2, dx = lane % 5 - 2;
+    const int delta = dy * (int)p.cols + dx;
+    const bool stacked = cm_kind(p) == PD_CM_MEAN_STACKED;
+    const uint32_t per_frame = cm_per_frame(p);
+#pragma unroll 4
+    for (int j = 0; j < kGatherHits; j++) {
+        const uint32_t f = __shfl_sync(0xffffffffu, own_f, j);
+        const uint32_t px = __shfl_sync(0xffffffffu, own_px, j);
+        const uint32_t m = __shfl_sync(0xffffffffu, own_m, j);
+        const uint32_t rc = __shfl_sync(0xffffffffu, own_rc, j);
+        if (h0 + j >= n || lane >= NPOS) continue;
+        const int r = (int)(rc >> 16) + dy, c = (int)(rc & 0xFFFFu) + dx;
+        float v = 0.0f;
+        if (r >= 0 && r < (int)p.rows && c >= 0 && c < (int)p.cols) {
+            const uint32_t g = px + (uint32_t)delta;
+            const uint32_t unit = m * p.units_per_module +
+                                  div16((uint32_t)r, dv.unit_rows) * p.units_per_row +
+                                  div16((uint32_t)c, dv.unit_cols);
+            const float* cmf = cm + (size_t)f * per_frame;
+            const uint16_t w = __ldg(raw + (size_t)f * p.frame_px + g);
+            float e;
+            if (MG) {
+                e = pd::mg_energy(mg, p.frame_px, w, g, cmf[unit]);
+            } else {
+                const float d = __fsub_rn(__uint2float_rn(w), __ldg(p.ped + g));
+                const float ig = __ldg(p.inv_gain + g);
+                if (stacked)
+                    e = pd::energy<true>(cm_after_gain(p), d, ig, cmf[unit],
+                                         cmf[p.units_per_frame + (size_t)m * p.rows + r],
+                                         cmf[p.units_per_frame + (size_t)p.n_modules * p.rows +
+                                             (size_t)m * p.cols + c]);
+                else
+                    e = pd::energy<false>(cm_after_gain(p), d, ig, cmf[unit], 0.0f, 0.0f);
+            }
+            v = __fdiv_rn(e, p.photon_kev);
         }
-        v = __fdiv_rn(e, p.photon_kev);
+        patches[(size_t)(h0 + j) * NPOS + lane] = v;
     }
-    patches[(size_t)h * NPOS + lane] = v;
 }
 
 // Replace count and (dx, dy) of hits the network is confident about; keep
@@ -338,14 +371,15 @@ cudaError_t launch_gather(const ChainParams& p, const uint16_t* raw, uint32_t fr
                           const float* cm, const pd_hit* hits, uint32_t n, float* patches,
                           cudaStream_t s, const MultiGain* mg) {
     if (!n) return cudaSuccess;
-    const uint32_t per = 8;  // hits per 256-thread block (one warp each)
+    const uint32_t per = 8 * kGatherHits;  // hits per 256-thread block
     const MultiGain m = mg ? *mg : MultiGain{};
+    auto magic = [](uint32_t d) { return d > 1 ? (uint32_t)(((1ull << 32) + d - 1) / d) : 0u; };
+    const GatherDiv dv{magic(p.unit_rows), magic(p.unit_cols)};
+    const unsigned blocks = n / per + (n % per != 0);
     if (mg)
-        gather_kernel<true><<<(n + per - 1) / per, 256, 0, s>>>(p, raw, frame_base, cm, hits, n,
-                                                              patches, m);
+        gather_kernel<true><<<blocks, 256, 0, s>>>(p, raw, frame_base, cm, hits, n, patches, m, dv);
     else
-        gather_kernel<false><<<(n + per - 1) / per, 256, 0, s>>>(p, raw, frame_base, cm, hits, n,
-                                                               patches, m);
+        gather_kernel<false><<<blocks, 256, 0, s>>>(p, raw, frame_base, cm, hits, n, patches, m, dv);
     return cudaGetLastError();
 }
 }  // namespace pd
