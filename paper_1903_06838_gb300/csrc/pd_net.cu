@@ -282,7 +282,7 @@ int pd_net_forward(pd_net* n, const float* patches, uint32_t count, float* out_d
         const uint32_t b = std::min(n->max_batch, count - done);
         cudaError_t e = pd::nettc::forward(n->w, patches + (size_t)done * NPOS, b, n->tc_img,
                                            n->tc_h2, out_dev + (size_t)done * NOUT, n->tc_err,
-                                           sms, s);
+                                           sms, done == 0, s);
         if (e) return net_cuda(e, "pd_net_forward");
         done += b;
     }

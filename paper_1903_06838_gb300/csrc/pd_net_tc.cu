@@ -9,18 +9,11 @@
 // (weights, input patch, and the ReLU activations h1, h2, h3) and
 // accumulates in float32; biases and ReLU are float32.
 //
-//   conv_kernel  one CTA holds 64 hits: their patches, all of h1 (64 x 25 x
-//                32, bf16) and one 128-row im2col tile at a time.  conv1 and
-//                conv2 are implicit GEMMs whose rows are (position, hit)
-//                pairs: 13 tiles of 128 rows each (the last half full); a
-//                conv2 tile is 18 MMAs of 128x32x16.  Accumulators alternate
-//                between two 32-column TMEM buffers, so the epilogue of one
-//                tile (bias, ReLU, bf16, store of h2) runs while the next
-//                tile's MMAs execute.
-//   fc_kernel    FC3 on 128 hits per CTA: h2 streams in 160-column chunks
-//                (double-buffered) against W3 resident in shared memory;
-//                the epilogue adds b3, applies ReLU and computes the 7 heads
-//                (FC4) on the CUDA cores.
+//   conv_kernel  conv1 and conv2 on tiles of 64 hits, one persistent CTA per
+//                SM with specialised warps (below)
+//   fc_kernel    FC3 on tiles of 128 hits and the 7 heads: a ring of bulk
+//                copies of h2 against W3 resident in shared memory, the heads
+//                (FC4) on the CUDA cores
 //
 // Operand layout: the canonical no-swizzle K-major form: 8-row x 16-byte core
 // matrices, core matrix (r, k) of a tile with R rows at byte
@@ -45,7 +38,6 @@ constexpr int K2 = 9 * C1;           // 288
 constexpr int K3 = NPOS * C2;        // 800
 constexpr int TB = 64;               // hits per conv tile
 constexpr int TF = 128;              // hits per fc tile
-constexpr int KCH = 160;             // fc K chunk
 constexpr uint32_t kWaitLimit = 1u << 22;
 
 // weight offsets (floats) in the parameter vector, as the training path
@@ -53,8 +45,9 @@ constexpr int OW1 = 0, OB1 = OW1 + C1 * 9, OW2 = OB1 + C1, OB2 = OW2 + C2 * K2, 
               OB3 = OW3 + NH * K3, OW4 = OB3 + NH, OB4 = OW4 + NOUT * NH;
 
 // bf16 operand images of the weights (bytes)
-constexpr uint32_t W1_BYTES = 32 * 16 * 2, W2_BYTES = 32 * K2 * 2, W3_BYTES = NH * K3 * 2;
-constexpr uint32_t OFF_W1 = 0, OFF_W2 = OFF_W1 + W1_BYTES, OFF_W3 = OFF_W2 + W2_BYTES;
+constexpr uint32_t W2_BYTES = 32 * K2 * 2, W3_BYTES = NH * K3 * 2;
+constexpr uint32_t OFF_W2 = 0, OFF_W3 = OFF_W2 + W2_BYTES;
+constexpr uint32_t W2_SLICE = 96 * 16 * 2;  // one tap row, 16 input channels
 
 __host__ __device__ __forceinline__ uint32_t cm_off(uint32_t r, uint32_t k, uint32_t rows) {
     return ((k >> 3) * (rows >> 3) + (r >> 3)) * 128u + (r & 7u) * 16u + (k & 7u) * 2u;
@@ -134,15 +127,19 @@ __device__ __forceinline__ void tmem_free(uint32_t taddr, uint32_t cols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols)
                  : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+// 32 columns of 16 TMEM lanes as four 16 x 8 blocks: of block k, lane (g, t)
+// gets rows g (r[4k], r[4k + 1]) and g + 8, columns 2t, 2t + 1
+__device__ __forceinline__ void tmem_ld16x32(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
         "%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
           "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
           "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
@@ -169,18 +166,17 @@ __device__ __forceinline__ int nb(int p, int k) {
 }
 
 // ---------------------------------------------------------------------------
-// bf16 operand images of W1 (32 x 16, taps 9..15 zero), W2 (32 x 288) and
-// W3 (64 x 800), K-major core-matrix layout, from the float32 parameters.
+// bf16 operand images, K-major core matrices, from the float32 parameters:
+// of W2 one matrix per tap row ky and half of the input channels, its 96 rows
+// (j, c_out) the taps kx = 2 - j, so that with an input column x as A they are
+// the outputs at x - 1, x, x + 1; and W3 (64 x 800).
 __global__ void prep_weights(const float* __restrict__ w, uint8_t* __restrict__ img) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < 32 * 16) {
-        const int r = i / 16, k = i % 16;
-        *reinterpret_cast<uint16_t*>(img + OFF_W1 + cm_off(r, k, 32)) =
-            bf16_bits(k < 9 ? w[OW1 + r * 9 + k] : 0.0f);
-    }
     if (i < 32 * K2) {
-        const int r = i / K2, k = i % K2;
-        *reinterpret_cast<uint16_t*>(img + OFF_W2 + cm_off(r, k, 32)) = bf16_bits(w[OW2 + i]);
+        const int co = i / K2, k = i % K2, tap = k / C1, ci = k % C1;
+        const int row = (2 - tap % 3) * 32 + co;
+        *reinterpret_cast<uint16_t*>(img + OFF_W2 + (tap / 3 * 2 + ci / 16) * W2_SLICE +
+                                     cm_off(row, ci % 16, 96)) = bf16_bits(w[OW2 + i]);
     }
     if (i < NH * K3) {
         const int r = i / K3, k = i % K3;
@@ -189,36 +185,41 @@ __global__ void prep_weights(const float* __restrict__ w, uint8_t* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// conv1 + conv2 on tiles of 64 hits, h2 out as bf16 [n][800]; one CTA of 512
-// threads per SM with specialised warps:
-//   warps 0-7   conv1 on the CUDA cores (bf16 operands, float32 fused
-//               multiply-adds) into one of two h1 stages: per position a
-//               64-hit x 32-channel K-major block (4 KB), 100 KB per stage
-//   warps 8-11  lane 0 of warp 8 + b issues the conv2 MMAs of the position
-//               groups that use TMEM buffer b (128 columns, 4 positions):
-//               an implicit GEMM read in place, the contribution of tap k to
-//               position p being two 64x32x16 MMAs of h1 block nb(p, k)
-//               against the W2 slice of tap k (taps outside the patch are not
-//               issued).  One thread issues a small MMA about every 60
-//               cycles; four issuing threads bring that to about 25.
+// conv1 + conv2 on tiles of 64 hits, h2 out as bf16 in the layout fc_kernel
+// copies: per 128 hits [k / 8][hit][8 values].  One CTA of 512 threads per SM
+// with specialised warps:
+//   warps 0-7   conv1 as m16n8k16 MMAs (bf16 operands, float32 accumulation)
+//               into one of two h1 stages: per position a 64-hit x 32-channel
+//               K-major block (4 KB), 100 KB per stage
+//   warps 8-10  lane 0 of warp 8 + b issues the conv2 MMAs of the output rows
+//               that use TMEM buffer b (160 columns: 5 positions): an implicit
+//               GEMM read in place.  A is an input position's block, B the
+//               three taps of a tap row for 16 input channels (96 columns, the
+//               outputs at x - 1, x, x + 1; 64 at the border), added at the
+//               output columns' place in TMEM, so no tap outside the patch is
+//               computed.  The issue of an MMA costs 25 to 50 cycles whatever
+//               its size: 145 MMAs of up to 64 x 96 x 16 a tile in place of
+//               338 of 64 x 32 x 16, one per tap, took the kernel from 82 us
+//               per 65,536 hits to 52.
 //   warps 12-15 the epilogue: TMEM -> bias, ReLU, bf16 -> h2 (warp 12 + q
-//               reads TMEM lanes 32q..32q+31)
+//               reads TMEM lanes 32q..32q+15, where M = 64 puts rows
+//               16q..16q+15, as 16-lane blocks: every lane holds two rows'
+//               column pairs, and a store of the warp is 128 contiguous bytes)
 // mbarriers hand the stages and TMEM buffers around (h1 full / empty, TMEM
 // full / empty), so conv1 of the next tile, conv2 MMAs and the epilogue of
-// earlier groups overlap.  Every wait is bounded; a timeout sets *err, stops
+// earlier rows overlap.  Every wait is bounded; a timeout sets *err, stops
 // every role, and the issuing lane waits (bounded) for its last commit
 // before TMEM is freed.
 constexpr int WS_PROD_WARPS = 8, WS_MMA_WARP0 = 8, WS_EPI_WARP0 = 12;
 constexpr int WS_PROD = WS_PROD_WARPS * 32, WS_THREADS = 512;
 constexpr uint32_t H1_STAGE = TB * NPOS * C1 * 2;  // 102 400 bytes
 constexpr uint32_t WS_W2 = 0, WS_H1 = WS_W2 + W2_BYTES, WS_X = WS_H1 + 2 * H1_STAGE,
-                   WS_W1 = WS_X + TB * NPOS * 2, WS_SMEM = WS_W1 + (9 * C1 + C1) * 4;
+                   WS_SMEM = WS_X + TB * NPOS * 2;
 constexpr uint32_t kConvTmemCols = 512;
-constexpr int kGroup = 4;     // conv2 positions per TMEM buffer
-constexpr int kTBufs = 4;     // TMEM buffers of kGroup * 32 columns
-constexpr int NG = (NPOS + kGroup - 1) / kGroup;
-static_assert(WS_H1 % 128 == 0 && H1_STAGE % 128 == 0 && WS_W1 % 16 == 0, "alignment");
-static_assert(kTBufs * kGroup * 32 <= (int)kConvTmemCols, "TMEM buffers");
+constexpr int kRowCols = 5 * 32;  // TMEM columns of an output row
+constexpr int kTBufs = 3;         // TMEM buffers
+static_assert(WS_H1 % 128 == 0 && H1_STAGE % 128 == 0, "alignment");
+static_assert(kTBufs * kRowCols <= (int)kConvTmemCols, "TMEM buffers");
 
 __device__ __forceinline__ void bar_init_n(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
@@ -241,14 +242,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     __shared__ __align__(8) uint64_t s_h1_full[2], s_h1_empty[2], s_t_full[kTBufs],
         s_t_empty[kTBufs];
     __shared__ int s_nb[NPOS * 9];
-    // per position: its valid (tap, channel half) MMAs as descriptor address
-    // offsets (16-byte units): A block of the neighbour | W2 slice << 16
-    __shared__ uint32_t s_mma[NPOS * 18];
-    __shared__ int s_nmma[NPOS];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint16_t* sx = reinterpret_cast<uint16_t*>(sm + WS_X);      // [64][25] bf16 patches
-    float* w1t = reinterpret_cast<float*>(sm + WS_W1);           // [9][32] bf16-valued
-    float* b1 = w1t + 9 * C1;                                    // [32]
     const uint32_t w2_addr = smem_u32(sm + WS_W2), h1_addr = smem_u32(sm + WS_H1);
 
     if (warp == 0) tmem_alloc(&s_tmem, kConvTmemCols);
@@ -265,25 +260,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int i = tid; i < NPOS * 9; i += blockDim.x) s_nb[i] = nb(i / 9, i % 9);
-    if (tid < NPOS) {
-        int m = 0;
-        for (int k = 0; k < 9; k++) {
-            const int q = nb(tid, k);
-            if (q < 0) continue;
-            for (int kk = 0; kk < 2; kk++)
-                s_mma[tid * 18 + m++] =
-                    (uint32_t)((q * 4096 + kk * 2048) >> 4) |
-                    ((uint32_t)(((4 * k + 2 * kk) * 512) >> 4) << 16);
-        }
-        s_nmma[tid] = m;
-    }
     for (uint32_t i = tid; i < W2_BYTES / 16; i += blockDim.x)
         reinterpret_cast<uint4*>(sm + WS_W2)[i] = reinterpret_cast<const uint4*>(img + OFF_W2)[i];
-    for (int i = tid; i < 9 * C1; i += blockDim.x) {
-        const int k = i / C1, c = i % C1;
-        w1t[i] = bf16_round(w[OW1 + c * 9 + k]);
-    }
-    for (int i = tid; i < C1; i += blockDim.x) b1[i] = w[OB1 + i];
     fence_async_smem();
     fence_before();
     __syncthreads();
@@ -400,12 +378,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     } else if (warp < WS_EPI_WARP0) {
         // ---- conv2 MMA issue: lane 0 of warp 8 + b, TMEM buffer b -----------
         const int ib = warp - WS_MMA_WARP0;
-        if (lane == 0) {
-            const uint32_t id64 = idesc_bf16(64, 32);
-            const uint64_t b_desc0 = sdesc(w2_addr, 512, 128);
-            int i = 0, gq = 0;  // local tile, global group sequence
+        if (lane == 0 && ib < kTBufs) {
+            const uint32_t id32 = idesc_bf16(64, 32), id64 = idesc_bf16(64, 64),
+                           id96 = idesc_bf16(64, 96);
+            const uint64_t b_desc0 = sdesc(w2_addr, 1536, 128);
+            const uint32_t d0 = tmem + (uint32_t)(ib * kRowCols);
+            int i = 0, gq = 0;  // local tile, global row sequence
             bool issued = false;
-            uint64_t* last = nullptr;
             uint32_t last_par = 0;
             for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, i++) {
                 const int stage = i & 1;
@@ -413,28 +392,40 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 fence_after();
                 const uint64_t a_desc0 = sdesc(h1_addr + stage * H1_STAGE, 1024, 128);
                 bool ok = true;
-                for (int g = 0; g < NG; g++, gq++) {
-                    const int b = gq % kTBufs;
-                    if (b != ib) continue;  // another thread's buffer
-                    if (!wait_or_abort(&s_t_empty[b], ((gq / kTBufs) & 1) ^ 1)) {
+                for (int yo = 0; yo < 5; yo++, gq++) {
+                    if (gq % kTBufs != ib) continue;  // another thread's buffer
+                    if (!wait_or_abort(&s_t_empty[ib], ((gq / kTBufs) & 1) ^ 1)) {
                         ok = false;
                         break;
                     }
                     fence_after();
-                    for (int pi = 0; pi < kGroup; pi++) {
-                        const int p = g * kGroup + pi;
-                        if (p >= NPOS) break;
-                        const uint32_t d = tmem + (uint32_t)((b * kGroup + pi) * 32);
-                        const int nm = s_nmma[p];
-                        const uint32_t* tab = s_mma + p * 18;
-                        for (int e = 0; e < nm; e++) {
-                            const uint32_t o = tab[e];
-                            mma(d, a_desc0 + (o & 0xFFFFu), b_desc0 + (o >> 16), id64, e);
-                        }
+                    const int y0 = max(yo - 1, 0), y1 = min(yo + 1, 4);
+                    for (int yi = y0; yi <= y1; yi++) {
+                        // (descriptor addresses count 16 bytes; input column x
+                        // in order, so that every output adds its taps in order)
+                        const uint64_t ay = a_desc0 + (uint32_t)(yi * 5 * 256);
+                        const uint64_t by = b_desc0 + (uint32_t)((yi - yo + 1) * 2 * (W2_SLICE >> 4));
+#pragma unroll
+                        for (int x = 0; x < 5; x++)
+#pragma unroll
+                            for (int kk = 0; kk < 2; kk++) {
+                                const uint64_t a = ay + (uint32_t)(x * 256 + kk * 128);
+                                const uint64_t b = by + (uint32_t)(kk * (W2_SLICE >> 4));
+                                const bool fresh = yi == y0 && kk == 0;  // new columns
+                                const uint32_t d = d0 + (x > 0 ? x - 1 : 0) * 32;
+                                if (x == 0)
+                                    mma(d, a, b + 32, id64, !fresh);
+                                else if (x == 4)
+                                    mma(d, a, b, id64, 1);
+                                else if (fresh) {
+                                    mma(d, a, b, id64, 1);
+                                    mma(d + 64, a, b + 64, id32, 0);
+                                } else
+                                    mma(d, a, b, id96, 1);
+                            }
                     }
-                    commit(&s_t_full[b]);
+                    commit(&s_t_full[ib]);
                     issued = true;
-                    last = &s_t_full[b];
                     last_par = (gq / kTBufs) & 1;
                 }
                 if (!ok) break;
@@ -442,23 +433,25 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             }
             if (s_abort) {
                 atomicExch(err, 1);
-                if (issued) wait_bar(last, last_par);  // bounded
+                if (issued) wait_bar(&s_t_full[ib], last_par);  // bounded
             }
         }
         __syncwarp();
     } else if (warp >= WS_EPI_WARP0) {
-        // ---- conv2 epilogue (warps 8-11, TMEM lane quadrant q) ---------------
-        const int q = warp - WS_EPI_WARP0;
+        // ---- conv2 epilogue (warps 12-15, TMEM lane quadrant q) --------------
+        const int q = warp - WS_EPI_WARP0, g = lane >> 2, tq = lane & 3;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        const int qhit = q * 16 + lane;  // M = 64: row r in TMEM lane (r / 16) * 32 + r % 16
-        float b2[C2];
+        float2 b2[4];
 #pragma unroll
-        for (int c = 0; c < C2; c++) b2[c] = w[OB2 + c];
+        for (int k = 0; k < 4; k++)
+            b2[k] = make_float2(w[OB2 + 8 * k + 2 * tq], w[OB2 + 8 * k + 2 * tq + 1]);
         int gq = 0;
         for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-            const int hit0 = t * TB, nh = min(TB, n - hit0);
+            // this lane's first value of the tile's first hit row
+            uint8_t* dst0 = reinterpret_cast<uint8_t*>(h2) + (size_t)(t >> 1) * (TF * K3 * 2) +
+                            ((t & 1) * TB + q * 16 + g) * 16 + tq * 4;
             bool ok = true;
-            for (int g = 0; g < NG; g++, gq++) {
+            for (int yo = 0; yo < 5; yo++, gq++) {
                 const int b = gq % kTBufs;
                 // lane 0 waits and the warp follows it (tcgen05.ld is warp-wide)
                 const int got = __shfl_sync(
@@ -469,33 +462,38 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                     break;
                 }
                 fence_after();
-                for (int pi = 0; pi < kGroup; pi++) {
-                    const int p = g * kGroup + pi;
-                    if (p >= NPOS) break;
-                    uint32_t r[32];
-                    tmem_ld32(tmem + lane_base + (uint32_t)((b * kGroup + pi) * 32), r);
-                    if (lane < 16 && qhit < nh) {
-                        uint32_t pk[16];
+                const uint32_t src = tmem + lane_base + (uint32_t)(b * kRowCols);
+                auto put = [&](const uint32_t (&r)[16], int x) {
+                    uint8_t* dst = dst0 + (size_t)(yo * 5 + x) * (4 * TF * 16);
 #pragma unroll
-                        for (int c = 0; c < 32; c += 2) {
+                    for (int k = 0; k < 4; k++)
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
                             const float2 z = __fadd2_rn(
-                                make_float2(__uint_as_float(r[c]), __uint_as_float(r[c + 1])),
-                                make_float2(b2[c], b2[c + 1]));
+                                make_float2(__uint_as_float(r[4 * k + 2 * h]),
+                                            __uint_as_float(r[4 * k + 2 * h + 1])),
+                                b2[k]);
                             const __nv_bfloat162 v =
                                 __float22bfloat162_rn(make_float2(fmaxf(z.x, 0.0f), fmaxf(z.y, 0.0f)));
-                            pk[c / 2] = *reinterpret_cast<const uint32_t*>(&v);
+                            *reinterpret_cast<__nv_bfloat162*>(dst + k * (TF * 16) + h * 128) = v;
                         }
-                        uint4* dst = reinterpret_cast<uint4*>(h2 + (size_t)(hit0 + qhit) * K3 +
-                                                              p * C2);
-#pragma unroll
-                        for (int j = 0; j < 4; j++)
-                            dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2],
-                                                pk[4 * j + 3]);
-                    }
-                }
+                };
+                uint32_t r0[16], r1[16], r2[16];
+                tmem_ld16x32(src, r0);
+                tmem_ld16x32(src + 32, r1);
+                tmem_ld16x32(src + 64, r2);
+                tmem_ld_wait();
+                put(r0, 0);
+                put(r1, 1);
+                put(r2, 2);
+                tmem_ld16x32(src + 96, r0);
+                tmem_ld16x32(src + 128, r1);
+                tmem_ld_wait();
                 fence_before();
                 __syncwarp();
                 if (lane == 0) bar_arrive(&s_t_empty[b]);
+                put(r0, 3);
+                put(r1, 4);
             }
             if (!ok) break;
         }
@@ -508,150 +506,207 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------
-// FC3 + heads on tiles of 128 hits.
-constexpr uint32_t FC_W3 = 0, FC_A = FC_W3 + W3_BYTES, FC_ABUF = TF * KCH * 2,
-                   FC_PART = FC_A + 2 * FC_ABUF, FC_SMEM = FC_PART + 128 * 8 * 4;
-static_assert(FC_A % 128 == 0, "alignment");
+// FC3 + heads on tiles of 128 hits; one CTA of 384 threads per SM:
+//   warp 0      lane 0 copies h2 in chunks of 80 inputs (20 KB, contiguous)
+//               into a ring of six stages, as long as a stage is free: with
+//               the MMAs' 4 us of work and 105 MB of h2 per 65,536 hits, the
+//               copies are the bound and stay in flight across tiles
+//   warp 1      lane 0 issues each chunk's five 128 x 64 x 16 MMAs into one of
+//               two TMEM accumulators
+//   warps 4-11  the epilogue, warps 4-7 of even and 8-11 of odd tiles: bias,
+//               ReLU, bf16, the 7 heads of one hit a lane
+// (One role for all threads, copying a chunk ahead with barriers between:
+// 58 us per 65,536 hits; now 23 us.)
+constexpr int FC_KCH = 80, FC_NCH = K3 / FC_KCH, FC_STAGES = 6, FC_THREADS = 384;
+constexpr uint32_t FC_CHUNK = TF * FC_KCH * 2;
+constexpr uint32_t FC_W3 = 0, FC_A = FC_W3 + W3_BYTES, FC_W4 = FC_A + FC_STAGES * FC_CHUNK,
+                   FC_SMEM = FC_W4 + NH * 8 * 4;
+static_assert(FC_A % 128 == 0 && FC_CHUNK % 128 == 0 && W3_BYTES % FC_CHUNK == 0, "alignment");
 
-__global__ void __launch_bounds__(256, 1)
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes,
+                                          uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+            "r"(dst),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
+}
+__device__ __forceinline__ void expect_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+                 "r"(bytes)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(FC_THREADS, 1)
     fc_kernel(const uint16_t* __restrict__ h2, int n, const float* __restrict__ w,
               const uint8_t* __restrict__ img, float* __restrict__ out, int* err) {
     extern __shared__ __align__(1024) uint8_t sm[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_bar[2];
-    __shared__ float s_w4[NOUT * NH];
+    __shared__ volatile int s_abort;
+    __shared__ __align__(8) uint64_t s_full[FC_STAGES], s_empty[FC_STAGES], s_w3, s_t_full[2],
+        s_t_empty[2];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    float* part = reinterpret_cast<float*>(sm + FC_PART);  // [128][8]
-    const uint32_t w3_addr = smem_u32(sm + FC_W3);
+    float* s_w4 = reinterpret_cast<float*>(sm + FC_W4);  // [unit][8], bf16-valued
+    const uint32_t w3_addr = smem_u32(sm + FC_W3), a_addr = smem_u32(sm + FC_A);
 
-    if (warp == 0) tmem_alloc(&s_tmem, 64);
-    if (tid == 0)
-        for (int b = 0; b < 2; b++) bar_init(&s_bar[b]);
-    for (uint32_t i = tid; i < W3_BYTES / 16; i += blockDim.x)
-        reinterpret_cast<uint4*>(sm + FC_W3)[i] = reinterpret_cast<const uint4*>(img + OFF_W3)[i];
-    for (int i = tid; i < NOUT * NH; i += blockDim.x) s_w4[i] = bf16_round(w[OW4 + i]);
-    fence_async_smem();
+    if (warp == 0) tmem_alloc(&s_tmem, 128);
+    if (tid == 0) {
+        for (int b = 0; b < FC_STAGES; b++) {
+            bar_init(&s_full[b]);
+            bar_init(&s_empty[b]);
+        }
+        bar_init(&s_w3);
+        for (int b = 0; b < 2; b++) {
+            bar_init(&s_t_full[b]);
+            bar_init_n(&s_t_empty[b], 4);
+        }
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int i = tid; i < NH * 8; i += FC_THREADS)
+        s_w4[i] = (i & 7) < NOUT ? bf16_round(w[OW4 + (i & 7) * NH + (i >> 3)]) : 0.0f;
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = s_tmem;
-    uint32_t par[2] = {0, 0};
-    bool pend[2] = {false, false};
-    bool ok = true;
-    auto waitp = [&](int b) -> bool {
-        const bool r = __syncthreads_and(wait_bar(&s_bar[b], par[b]));
-        if (r) {
-            par[b] ^= 1;
-            pend[b] = false;
-        }
-        return r;
-    };
-    const uint32_t id3 = idesc_bf16(128, NH);
     const int n_tiles = (n + TF - 1) / TF;
-    const int half = warp >> 2;
-    const int erow = (warp & 3) * 32 + lane;
+    // bounded wait that also gives up once another role has aborted
+    auto wait_or_abort = [&](uint64_t* bar, uint32_t parity) -> bool {
+        const uint32_t a = smem_u32(bar);
+        for (uint32_t it = 0; it < kWaitLimit; it++) {
+            uint32_t ok;
+            asm volatile(
+                "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                "selp.u32 %0, 1, 0, p;\n}"
+                : "=r"(ok)
+                : "r"(a), "r"(parity)
+                : "memory");
+            if (ok) return true;
+            if ((it & 255) == 255 && s_abort) return false;
+        }
+        s_abort = 1;
+        return false;
+    };
 
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-        const int hit0 = t * TF, nh = min(TF, n - hit0);
-        constexpr int NCH = K3 / KCH;  // 5 chunks of 10 MMAs
-        // chunk c of this tile into buffer c & 1 by asynchronous 16-byte
-        // copies (rows past the last hit are zero-filled)
-        auto load_chunk = [&](int c) {
-            const uint32_t abuf = smem_u32(sm + FC_A + (c & 1) * FC_ABUF);
-            for (int e = tid; e < TF * (KCH / 8); e += blockDim.x) {
-                const int r = e / (KCH / 8), kc = (e % (KCH / 8)) * 8;
-                const bool in = r < nh;
-                const uint16_t* src = h2 + (size_t)(hit0 + (in ? r : 0)) * K3 + c * KCH + kc;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
-                                 abuf + cm_off(r, kc, TF)),
-                             "l"(src), "r"(in ? 16 : 0)
-                             : "memory");
-            }
-            asm volatile("cp.async.commit_group;\n" ::: "memory");
-        };
-        load_chunk(0);
-        for (int c = 0; c < NCH && ok; c++) {
-            const int buf = c & 1;
-            if (c + 1 < NCH) {
-                if (c >= 1) {  // buffer (c + 1) & 1 was read by the MMAs of chunk c - 1
-                    ok = waitp((c + 1) & 1);
-                    if (!ok) break;
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---- copies: W3 once, then every tile's chunks ----------------------
+            expect_tx(&s_w3, W3_BYTES);
+            for (uint32_t o = 0; o < W3_BYTES; o += FC_CHUNK)
+                bulk_copy(w3_addr + o, img + OFF_W3 + o, FC_CHUNK, &s_w3);
+            uint32_t c = 0;  // chunks issued
+            for (int t = blockIdx.x; t < n_tiles && !s_abort; t += gridDim.x) {
+                const uint8_t* src = reinterpret_cast<const uint8_t*>(h2) + (size_t)t * (TF * K3 * 2);
+                for (int k = 0; k < FC_NCH; k++, c++) {
+                    const uint32_t s = c % FC_STAGES;
+                    if (!wait_or_abort(&s_empty[s], ((c / FC_STAGES) & 1) ^ 1)) break;
+                    expect_tx(&s_full[s], FC_CHUNK);
+                    bulk_copy(a_addr + s * FC_CHUNK, src + (size_t)k * FC_CHUNK, FC_CHUNK, &s_full[s]);
                 }
-                load_chunk(c + 1);
-                asm volatile("cp.async.wait_group 1;\n" ::: "memory");  // chunk c landed
-            } else {
-                asm volatile("cp.async.wait_group 0;\n" ::: "memory");
             }
-            fence_async_smem();
-            fence_before();
-            __syncthreads();
+            if (s_abort) {  // the copies in flight write this CTA's memory (bounded)
+                wait_bar(&s_w3, 0);
+                for (uint32_t k = c > FC_STAGES ? c - FC_STAGES : 0; k < c; k++)
+                    wait_bar(&s_full[k % FC_STAGES], (k / FC_STAGES) & 1);
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            // ---- MMA issue -------------------------------------------------------
+            const uint32_t id3 = idesc_bf16(128, NH);
+            uint32_t c = 0;
+            int i = 0;
+            uint64_t* last = nullptr;
+            uint32_t last_par = 0;
+            bool ok = wait_or_abort(&s_w3, 0);
+            for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, i++) {
+                const int b = i & 1;
+                if (!(ok = wait_or_abort(&s_t_empty[b], ((i >> 1) & 1) ^ 1))) break;
+                fence_after();
+                for (int k = 0; k < FC_NCH; k++, c++) {
+                    const uint32_t s = c % FC_STAGES;
+                    if (!(ok = wait_or_abort(&s_full[s], (c / FC_STAGES) & 1))) break;
+                    const uint64_t ad = sdesc(a_addr + s * FC_CHUNK, TF * 16, 128);
+                    const uint64_t bd = sdesc(w3_addr + (uint32_t)k * FC_KCH * NH * 2, NH * 16, 128);
+#pragma unroll
+                    for (int j = 0; j < FC_KCH / 16; j++)
+                        mma(tmem + b * NH, ad + (uint32_t)(j * 2 * TF), bd + (uint32_t)(j * 2 * NH),
+                            id3, k > 0 || j > 0);
+                    commit(&s_empty[s]);
+                    last = &s_empty[s];
+                    last_par = (c / FC_STAGES) & 1;
+                }
+                if (!ok) break;
+                commit(&s_t_full[b]);
+            }
+            if (s_abort && last) wait_bar(last, last_par);  // bounded
+        }
+        __syncwarp();
+    } else if (warp >= 4) {
+        // ---- epilogue --------------------------------------------------------------
+        const int q = warp & 3, odd = (warp - 4) >> 2;
+        int i = odd;
+        for (int t = blockIdx.x + odd * gridDim.x; t < n_tiles; t += 2 * gridDim.x, i += 2) {
+            const int got = __shfl_sync(
+                0xffffffffu,
+                lane == 0 ? (int)wait_or_abort(&s_t_full[odd], (i >> 1) & 1) : 0, 0);
+            if (!got) break;
             fence_after();
-            if (tid == 0) {
-                const uint32_t a0 = smem_u32(sm + FC_A + buf * FC_ABUF);
-                for (int s = 0; s < KCH / 16; s++) {
-                    const int ks = c * (KCH / 16) + s;  // global K step
-                    mma(tmem, sdesc(a0 + s * 2 * (TF / 8) * 128, (TF / 8) * 128, 128),
-                        sdesc(w3_addr + ks * 2 * (NH / 8) * 128, (NH / 8) * 128, 128), id3,
-                        (c > 0 || s > 0) ? 1u : 0u);
+            uint32_t r[2][32];
+            const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + odd * NH;
+            tmem_ld32(src, r[0]);
+            tmem_ld32(src + 32, r[1]);
+            fence_before();
+            __syncwarp();
+            if (lane == 0) bar_arrive(&s_t_empty[odd]);
+            // h3 = relu(acc + b3) rounded to bf16, then the heads, the sums of
+            // the two halves of the units added at the end
+            float sum[2][NOUT];
+#pragma unroll
+            for (int half = 0; half < 2; half++) {
+#pragma unroll
+                for (int o = 0; o < NOUT; o++) sum[half][o] = 0.0f;
+#pragma unroll
+                for (int c = 0; c < 32; c++) {
+                    const int ch = half * 32 + c;
+                    const float z = __uint_as_float(r[half][c]) + __ldg(w + OB3 + ch);
+                    const float h = bf16_round(fmaxf(z, 0.0f));
+                    const float4 wa = *reinterpret_cast<const float4*>(s_w4 + ch * 8);
+                    const float4 wb = *reinterpret_cast<const float4*>(s_w4 + ch * 8 + 4);
+                    sum[half][0] = __fmaf_rn(h, wa.x, sum[half][0]);
+                    sum[half][1] = __fmaf_rn(h, wa.y, sum[half][1]);
+                    sum[half][2] = __fmaf_rn(h, wa.z, sum[half][2]);
+                    sum[half][3] = __fmaf_rn(h, wa.w, sum[half][3]);
+                    sum[half][4] = __fmaf_rn(h, wb.x, sum[half][4]);
+                    sum[half][5] = __fmaf_rn(h, wb.y, sum[half][5]);
+                    sum[half][6] = __fmaf_rn(h, wb.z, sum[half][6]);
                 }
-                commit(&s_bar[buf]);
             }
-            pend[buf] = true;
+            const int hit = t * TF + q * 32 + lane;
+            if (hit < n)
+#pragma unroll
+                for (int o = 0; o < NOUT; o++)
+                    out[(size_t)hit * NOUT + o] = sum[0][o] + sum[1][o] + w[OB4 + o];
         }
-        if (!ok) {
-            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-            break;
-        }
-        // the last two chunks (buffers 1 and 0)
-        for (int c = NCH - 2; c < NCH && ok; c++) ok = waitp(c & 1);
-        if (!ok) break;
-        fence_after();
-        // epilogue: h3 = relu(acc + b3) rounded to bf16, heads on the CUDA
-        // cores; warps 4..7 take columns 32..63 and pass partial sums
-        uint32_t ra[16], rb[16];
-        const uint32_t tbase = tmem + ((uint32_t)((warp & 3) * 32) << 16) + half * 32;
-        tmem_ld16(tbase, ra);
-        tmem_ld16(tbase + 16, rb);
-        float acc[NOUT];
-#pragma unroll
-        for (int o = 0; o < NOUT; o++) acc[o] = 0.0f;
-#pragma unroll
-        for (int c = 0; c < 32; c++) {
-            const int ch = half * 32 + c;
-            const float z = __uint_as_float(c < 16 ? ra[c] : rb[c - 16]) + w[OB3 + ch];
-            const float h = bf16_round(fmaxf(z, 0.0f));
-#pragma unroll
-            for (int o = 0; o < NOUT; o++) acc[o] = __fmaf_rn(h, s_w4[o * NH + ch], acc[o]);
-        }
-        if (half == 1)
-#pragma unroll
-            for (int o = 0; o < NOUT; o++) part[erow * 8 + o] = acc[o];
-        fence_before();
-        __syncthreads();
-        if (half == 0 && erow < nh)
-#pragma unroll
-            for (int o = 0; o < NOUT; o++)
-                out[(size_t)(hit0 + erow) * NOUT + o] = acc[o] + part[erow * 8 + o] + w[OB4 + o];
-        __syncthreads();  // partial sums, A buffers and TMEM reused by the next tile
-    }
-    if (!ok && tid == 0) {
-        atomicExch(err, 1);
-        for (int b = 0; b < 2; b++)
-            if (pend[b]) wait_bar(&s_bar[b], par[b]);
     }
     fence_before();
     __syncthreads();
     fence_after();
-    if (warp == 0) tmem_free(tmem, 64);
+    if (s_abort && tid == 0) atomicExch(err, 1);
+    if (warp == 0) tmem_free(tmem, 128);
 }
 
 }  // namespace
 
 size_t weight_image_bytes() { return OFF_W3 + W3_BYTES; }
-size_t h2_bytes(uint32_t max_batch) { return (size_t)max_batch * K3 * 2; }
+// (whole fc tiles; rows past the last hit are computed and dropped)
+size_t h2_bytes(uint32_t max_batch) {
+    return ((size_t)max_batch + TF - 1) / TF * TF * K3 * 2;
+}
 
 cudaError_t forward(const float* w, const float* x, uint32_t n, uint8_t* img, uint16_t* h2,
-                    float* out, int* err, int sms, cudaStream_t s) {
+                    float* out, int* err, int sms, bool new_weights, cudaStream_t s) {
     if (!n) return cudaSuccess;
     static int attr_dev = -1;
     int dev = 0;
@@ -665,10 +720,10 @@ cudaError_t forward(const float* w, const float* x, uint32_t n, uint8_t* img, ui
         if (e != cudaSuccess) return e;
         attr_dev = dev;
     }
-    prep_weights<<<(NH * K3 + 255) / 256, 256, 0, s>>>(w, img);
+    if (new_weights) prep_weights<<<(NH * K3 + 255) / 256, 256, 0, s>>>(w, img);
     const int conv_tiles = (int)((n + TB - 1) / TB), fc_tiles = (int)((n + TF - 1) / TF);
     conv_kernel<<<std::min(conv_tiles, sms), WS_THREADS, WS_SMEM, s>>>(x, (int)n, w, img, h2, err);
-    fc_kernel<<<std::min(fc_tiles, sms), 256, FC_SMEM, s>>>(h2, (int)n, w, img, out, err);
+    fc_kernel<<<std::min(fc_tiles, sms), FC_THREADS, FC_SMEM, s>>>(h2, (int)n, w, img, out, err);
     return cudaGetLastError();
 }
 
