@@ -967,6 +967,7 @@ int pd_set_tuning(pd_ctx* c, const pd_tuning* t) {
         if (pd::band_smem_bytes(c->params, rb, c->band_cfg.pitch) > 200 * 1024)
             return fail(PD_EINVAL, "band too tall for shared memory");
         c->band_cfg.rb = rb;
+        c->band_cfg.fit = rb == pd::make_band_config(c->params).rb;
         c->band_cfg.n_bands = (c->params.rows + rb - 1) / rb;
     }
     c->overlap = t->overlap ? 1 : 0;

@@ -1210,6 +1210,7 @@ BandConfig make_band_config(const ChainParams& p) {
     while (rb > 1 && band_smem_bytes(p, rb, bc.pitch) > 100 * 1024) rb--;
     bc.rb = rb;
     bc.n_bands = (p.rows + rb - 1) / rb;
+    bc.fit = true;
     return bc;
 }
 
@@ -1220,11 +1221,21 @@ size_t band_smem_bytes(const ChainParams& p, uint32_t rb, uint32_t pitch) {
            (size_t)(rb + 1) * ((p.cols + 31) / 32) * 4;     // seed bitmap
 }
 
-cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& bc, const uint16_t* raw,
+cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& cfg, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
                                 cudaStream_t stream, const MultiGain* mg) {
+    if (n_frames == 0) return cudaSuccess;
+    BandConfig bc = cfg;
+    const auto ctas_per_sm = [&] {
+        const size_t smem = band_smem_bytes(p, bc.rb, bc.pitch);
+        return (int)std::max<size_t>(1, std::min<size_t>((200 * 1024) / smem, 4));
+    };
+    if (bc.fit) {
+        bc.rb = fit_band_rows(p.rows, bc.rb, bc.ty, (uint64_t)n_frames * p.n_modules,
+                              (uint64_t)device_sm_count() * ctas_per_sm());
+        bc.n_bands = (p.rows + bc.rb - 1) / bc.rb;
+    }
     const unsigned long long n_tiles = (unsigned long long)n_frames * p.n_modules * bc.n_bands;
-    if (n_tiles == 0) return cudaSuccess;
     if (mg && bc.vec != 4) return cudaErrorInvalidValue;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -1240,9 +1251,7 @@ cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& bc, cons
     }
     const size_t smem = band_smem_bytes(p, bc.rb, bc.pitch);
     const unsigned threads = bc.tx * bc.ty;
-    int per_sm = (int)((200 * 1024) / std::max<size_t>(smem, 1));
-    per_sm = std::max(1, std::min(per_sm, 4));
-    unsigned long long grid = (unsigned long long)device_sm_count() * per_sm;
+    unsigned long long grid = (unsigned long long)device_sm_count() * ctas_per_sm();
     if (grid > n_tiles) grid = n_tiles;
     const bool st = cm_kind(p) == PD_CM_MEAN_STACKED;
     const MultiGain m = mg ? *mg : MultiGain{};

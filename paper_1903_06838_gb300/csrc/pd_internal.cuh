@@ -126,6 +126,9 @@ struct MatchedBank {
     // or null) holds them for every mask
     uint32_t all_binary;
     const uint8_t* vtab;
+    // taps under some F1, and those that every feature's F0 holds (positive
+    // F0 only): a hit has signal at one of the former, none at the latter
+    uint32_t some, clear;
 };
 
 // Per-call outputs (device pointers).

@@ -1433,6 +1433,8 @@ LeanConfig make_lean_config(const ChainParams& p, uint32_t rb, bool multigain) {
         const uint32_t nb = (p.rows + t.rb - 1) / t.rb;
         rb = (p.rows + nb - 1) / nb;
     }
+    // (an explicit height that is the default one is the default)
+    lc.fit = dflt || make_lean_config(p, 0, multigain).rb == rb;
     rb = std::min(rb, p.rows);
     // own rows per thread fit a 64-bit candidate mask (4 bits per row)
     while (rb > 1 && (rb + lc.ty - 1) / lc.ty > 16) rb--;
@@ -1495,11 +1497,20 @@ auto lean_pick(bool colbank, bool oneunit) {
 }
 }  // namespace
 
-cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& lc, const uint16_t* raw,
+cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& cfg, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
                                 uint32_t* err, cudaStream_t stream, const MultiGain* mg) {
+    if (n_frames == 0) return cudaSuccess;
+    LeanConfig lc = cfg;
+    if (lc.fit) {
+        const uint64_t slots = (uint64_t)device_sm_count() *
+                               (lc.ctas_per_sm ? lc.ctas_per_sm
+                                : lean_smem_bytes(p, lc) <= kLeanSmemTwo ? 2u : 1u);
+        lc.rb = fit_band_rows(p.rows, lc.rb, lc.ty, (uint64_t)n_frames * p.n_modules, slots);
+        lc.n_bands = (p.rows + lc.rb - 1) / lc.rb;
+        set_stage_periods(lc);
+    }
     const unsigned long long n_tiles = (unsigned long long)n_frames * p.n_modules * lc.n_bands;
-    if (n_tiles == 0) return cudaSuccess;
     int dev = 0;
     cudaGetDevice(&dev);
     if (g_attr_dev_lean != dev) {

@@ -93,6 +93,7 @@ struct LeanConfig {
     // seeds are tested
     uint32_t stage_t, stage_g, stage_bp;
     uint32_t wait_polls;  // polls of a staged copy or a tile's dependency (0: default)
+    bool fit;  // rb is the default: calls of few tiles take shorter bands
     bool ok;
 };
 

@@ -814,9 +814,16 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
                            const CallOut& out, cudaStream_t stream, const MultiGain* mg) {
     BandConfig bc;
     if (!mg && matched_band_config(p, &bc)) {
+        if (n_frames == 0) return cudaSuccess;
+        const auto ctas_per_sm = [&] {
+            const size_t per_cta = band_smem(p, bc.rb, bc.pitch) + sizeof(MatchedBank) + 1024;
+            return (int)std::max<size_t>(1, std::min<size_t>((228 * 1024) / per_cta, 2));
+        };
+        bc.rb = fit_band_rows(p.rows, bc.rb, bc.ty, (uint64_t)n_frames * p.n_modules,
+                              (uint64_t)device_sm_count() * ctas_per_sm());
+        bc.n_bands = (p.rows + bc.rb - 1) / bc.rb;
         const unsigned long long n_tiles =
             (unsigned long long)n_frames * p.n_modules * bc.n_bands;
-        if (n_tiles == 0) return cudaSuccess;
         int dev = 0;
         cudaGetDevice(&dev);
         if (g_attr_dev_mband != dev) {
@@ -828,10 +835,7 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
             g_attr_dev_mband = dev;
         }
         const size_t smem = band_smem(p, bc.rb, bc.pitch);
-        const size_t per_cta = smem + sizeof(MatchedBank) + 1024;
-        int per_sm = (int)((228 * 1024) / per_cta);
-        per_sm = std::max(1, std::min(per_sm, 2));
-        unsigned long long grid = (unsigned long long)device_sm_count() * per_sm;
+        unsigned long long grid = (unsigned long long)device_sm_count() * ctas_per_sm();
         if (grid > n_tiles) grid = n_tiles;
         const unsigned threads = bc.tx * bc.ty;
         if (cm_kind(p) == PD_CM_MEAN_STACKED)
