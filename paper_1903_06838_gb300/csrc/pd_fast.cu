@@ -595,7 +595,9 @@ struct BandShared {
 // raw rows of later tiles are asked of L2 ahead of their loads (the
 // single-context kernel; the batched one keeps its registers for the items'
 // parameters).
-template <int VEC, bool STACKED = false, bool MG = false, bool PREFETCH = false>
+// AG: the paper's order, d gain-corrected before the common mode, masked
+// pixels 0.
+template <int VEC, bool STACKED = false, bool MG = false, bool PREFETCH = false, bool AG = false>
 __device__ void stencil_band_run(const ChainParams& p, const uint16_t* __restrict__ raw,
                                  uint32_t frame_base, const CallOut& out, const BandConfig& bc,
                                  unsigned long long first, unsigned long long n_tiles,
@@ -700,7 +702,9 @@ __device__ void stencil_band_run(const ChainParams& p, const uint16_t* __restric
         //    are not histogrammed: their bins are clamped to the spare bin.
         if (active) {
             const int nrows = rows_here + 2;
-            constexpr int U = PD_BAND_UNROLL;
+            // (single pixels: few registers a row, and a module wider than
+            // half the block leaves one row lane, so more rows in flight)
+            constexpr int U = VEC == 1 ? 4 : PD_BAND_UNROLL;
             for (int rl0 = (int)ty; rl0 < nrows; rl0 += U * (int)TY) {
                 uint2 rr[U];
                 float4 pp[U], gg[U];
@@ -745,10 +749,16 @@ __device__ void stencil_band_run(const ChainParams& p, const uint16_t* __restric
                     const float ncmb = cmt[rl * p.units_per_row + ucb];
                     float e[VEC];
                     if (VEC == 4) {
-                        const float2 d01 = __fadd2_rn(raw_pair(rr[j].x), make_float2(pp[j].x, pp[j].y));
-                        const float2 d23 = __fadd2_rn(raw_pair(rr[j].y), make_float2(pp[j].z, pp[j].w));
+                        float2 d01 = __fadd2_rn(raw_pair(rr[j].x), make_float2(pp[j].x, pp[j].y));
+                        float2 d23 = __fadd2_rn(raw_pair(rr[j].y), make_float2(pp[j].z, pp[j].w));
                         const float2 n01 = make_float2(split > 0 ? ncma : ncmb, split > 1 ? ncma : ncmb);
                         const float2 n23 = make_float2(split > 2 ? ncma : ncmb, split > 3 ? ncma : ncmb);
+                        if (AG) {
+                            // (one by one: a packed product that only feeds a
+                            // packed sum is fused with it, and rounded once)
+                            d01 = make_float2(__fmul_rn(d01.x, gg[j].x), __fmul_rn(d01.y, gg[j].y));
+                            d23 = make_float2(__fmul_rn(d23.x, gg[j].z), __fmul_rn(d23.y, gg[j].w));
+                        }
                         float2 c01 = __fadd2_rn(d01, n01), c23 = __fadd2_rn(d23, n23);
                         if (STACKED) {
                             const float ncr = crt[rl];
@@ -757,8 +767,16 @@ __device__ void stencil_band_run(const ChainParams& p, const uint16_t* __restric
                             c23 = __fadd2_rn(__fadd2_rn(c23, make_float2(ncr, ncr)),
                                              make_float2(ncc[VEC > 2 ? 2 : 0], ncc[VEC > 3 ? 3 : 0]));
                         }
-                        float2 e01 = __fmul2_rn(c01, make_float2(gg[j].x, gg[j].y));
-                        float2 e23 = __fmul2_rn(c23, make_float2(gg[j].z, gg[j].w));
+                        float2 e01, e23;
+                        if (AG) {
+                            e01 = make_float2(gg[j].x == 0.0f ? 0.0f : c01.x,
+                                              gg[j].y == 0.0f ? 0.0f : c01.y);
+                            e23 = make_float2(gg[j].z == 0.0f ? 0.0f : c23.x,
+                                              gg[j].w == 0.0f ? 0.0f : c23.y);
+                        } else {
+                            e01 = __fmul2_rn(c01, make_float2(gg[j].x, gg[j].y));
+                            e23 = __fmul2_rn(c23, make_float2(gg[j].z, gg[j].w));
+                        }
                         if (MG && ((rr[j].x | rr[j].y) & (~mg.vmask << 16 | (~mg.vmask & 0xFFFFu)))) {
                             // words of a higher gain stage: that stage's pedestal
                             // and gain, no common mode; beyond the maps, 0
@@ -797,9 +815,14 @@ __device__ void stencil_band_run(const ChainParams& p, const uint16_t* __restric
                         atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u23.x), blo), bhi) - kMagicBits], 1u);
                         atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u23.y), blo), bhi) - kMagicBits], 1u);
                     } else {
-                        float c0 = __fadd_rn(__fadd_rn(__uint2float_rn(r1[j]), p1[j]), ncma);
+                        float c0 = __fadd_rn(__uint2float_rn(r1[j]), p1[j]);
+                        if (AG) c0 = __fmul_rn(c0, g1[j]);
+                        c0 = __fadd_rn(c0, ncma);
                         if (STACKED) c0 = __fadd_rn(__fadd_rn(c0, crt[rl]), ncc[0]);
-                        e[0] = __fmul_rn(c0, g1[j]);
+                        if (AG)
+                            e[0] = g1[j] == 0.0f ? 0.0f : c0;
+                        else
+                            e[0] = __fmul_rn(c0, g1[j]);
                         const float u = __fadd_rd(__fmaf_rn(e[0], p.hist_inv_w, p.hist_neg_lo_s),
                                                   kMagic);
                         atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u), blo), bhi) - kMagicBits], 1u);
@@ -962,14 +985,14 @@ __device__ void stencil_band_run(const ChainParams& p, const uint16_t* __restric
     }
 }
 
-template <int VEC, bool STACKED, bool MG = false>
+template <int VEC, bool STACKED, bool MG = false, bool AG = false>
 __global__ void __launch_bounds__(kBandThreads, 2)
     stencil_band_kernel(ChainParams p, const uint16_t* __restrict__ raw,
                         uint32_t frame_base, CallOut out, BandConfig bc,
                         unsigned long long n_tiles, MultiGain mg) {
     extern __shared__ __align__(16) uint32_t band_smem[];
     __shared__ BandShared bsh;
-    stencil_band_run<VEC, STACKED, MG, true>(p, raw, frame_base, out, bc, blockIdx.x, n_tiles,
+    stencil_band_run<VEC, STACKED, MG, true, AG>(p, raw, frame_base, out, bc, blockIdx.x, n_tiles,
                                              gridDim.x, band_smem, bsh, mg);
 }
 
@@ -1236,13 +1259,17 @@ cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& cfg, con
         bc.n_bands = (p.rows + bc.rb - 1) / bc.rb;
     }
     const unsigned long long n_tiles = (unsigned long long)n_frames * p.n_modules * bc.n_bands;
-    if (mg && bc.vec != 4) return cudaErrorInvalidValue;
+    if (mg && (bc.vec != 4 || cm_after_gain(p))) return cudaErrorInvalidValue;
     int dev = 0;
     cudaGetDevice(&dev);
     if (g_attr_dev_band != dev) {
         for (auto k : {stencil_band_kernel<4, false>, stencil_band_kernel<1, false>,
                        stencil_band_kernel<4, true>, stencil_band_kernel<1, true>,
-                       stencil_band_kernel<4, false, true>}) {
+                       stencil_band_kernel<4, false, true>,
+                       stencil_band_kernel<4, false, false, true>,
+                       stencil_band_kernel<1, false, false, true>,
+                       stencil_band_kernel<4, true, false, true>,
+                       stencil_band_kernel<1, true, false, true>}) {
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  200 * 1024);
             if (e != cudaSuccess) return e;
@@ -1260,6 +1287,11 @@ cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& cfg, con
              : bc.vec == 4       ? stencil_band_kernel<4, false>
              : st                ? stencil_band_kernel<1, true>
                                  : stencil_band_kernel<1, false>;
+    if (cm_after_gain(p))
+        k = bc.vec == 4 ? (st ? stencil_band_kernel<4, true, false, true>
+                              : stencil_band_kernel<4, false, false, true>)
+                        : (st ? stencil_band_kernel<1, true, false, true>
+                              : stencil_band_kernel<1, false, false, true>);
     k<<<(unsigned)grid, threads, smem, stream>>>(p, raw, frame_base, out, bc, n_tiles, m);
     return cudaGetLastError();
 }
