@@ -109,6 +109,13 @@ struct MatchedTap {
     uint16_t at;
     float v;
 };
+// A tap of the sums: its offset in the tile (as above, 16 bits; 5 i + j in the
+// upper ones until the band kernel rewrites it) and its weight in F1, F1dx and
+// F1dy, 0 where it is none of that filter's.
+struct alignas(16) MatchedSum {
+    uint32_t at;
+    float v1, vx, vy;
+};
 struct MatchedBank {
     uint32_t n_features;
     float nmin[PD_MAX_FEATURES];
@@ -118,9 +125,10 @@ struct MatchedBank {
     uint32_t m1[PD_MAX_FEATURES], m0[PD_MAX_FEATURES];
     uint32_t f1_unit[PD_MAX_FEATURES], f0_pos[PD_MAX_FEATURES];
     uint16_t off1[PD_MAX_FEATURES + 1], off0[PD_MAX_FEATURES + 1];
-    uint16_t offx[PD_MAX_FEATURES + 1], offy[PD_MAX_FEATURES + 1];
     MatchedTap t1[PD_MAX_FEATURES * 20], t0[PD_MAX_FEATURES * 20];
-    MatchedTap tx[PD_MAX_FEATURES * 20], ty[PD_MAX_FEATURES * 20];
+    // taps with a nonzero F1, F1dx or F1dy, for the three sums at once
+    uint16_t offs[PD_MAX_FEATURES + 1];
+    alignas(16) MatchedSum ts[PD_MAX_FEATURES * 20];
     // every feature binary (f1_unit and f0_pos): the valid features of a
     // pixel depend on its window mask alone, and vtab (device, 2^20 bytes,
     // or null) holds them for every mask

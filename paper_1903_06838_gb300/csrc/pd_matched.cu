@@ -35,14 +35,18 @@
 //
 // matched_band_kernel: the same per pixel on full-width bands of module rows
 // (single gain, raw - pedestal before the common mode), with the band
-// stencil's four-pixel vector loads and packed correction.  Each thread
-// stores the signal bits of its four pixels as one nibble (a pixel's window
-// mask is read from the nibbles of four rows), and a chunk with signal marks
-// the pixels whose windows it lies in on a bitmap of the band, from which
-// the candidate list is built.  The valid features of every candidate come
-// first (for a bank of binary features, from a table indexed by the window
-// mask); the sums then run over a second list of the candidates with a valid
-// feature, so that they keep every lane busy.
+// stencil's four-pixel vector loads and packed correction.  The signal bits of
+// the band go to a bitmap of 32 columns a word, and one thread per word finds
+// the pixels that may be hits, 32 at a time: a hit has a valid feature with
+// signal under its F1, so some tap of any F1 sees signal, and every tap that
+// all features' F0 share (those with positive taps) sees none.  The valid
+// features of these candidates come next (for a bank of binary features, from
+// a table indexed by the window mask); the sums then run over a second list of
+// the candidates with a valid feature, so that they keep every lane busy.
+// (Every pixel whose window held any signal was a candidate before: a quarter
+// of all at an occupancy of 0.5 %, each marked with up to eight shared atomics
+// and looked up in the table; 64 frames of 32 x 185 x 388: 556 -> 424 us,
+// with bands of 47 rows in place of 31 and one list of taps for the three sums.)
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -76,7 +80,7 @@ __device__ __forceinline__ uint32_t hist_bin(float v, float neg_lo_s, float inv_
 // and npix (the signal pixels under the first valid feature's F1), as
 // described above.
 __device__ __forceinline__ uint32_t valid_features(const MatchedBank& sb, const float* w,
-                                                   uint32_t win) {
+                                                   uint32_t win, float thr) {
     if (sb.vtab) return sb.vtab[win];
     uint32_t valid = 0;
     for (uint32_t ft = 0; ft < sb.n_features; ft++) {
@@ -86,7 +90,7 @@ __device__ __forceinline__ uint32_t valid_features(const MatchedBank& sb, const 
         } else {
             float over = 0.0f;
             for (uint32_t k = sb.off0[ft]; k < sb.off0[ft + 1]; k++)
-                if (w[sb.t0[k].at] > 0.0f) over = __fadd_rn(over, sb.t0[k].v);
+                if (w[sb.t0[k].at] > thr) over = __fadd_rn(over, sb.t0[k].v);
             clear = over == 0.0f;
         }
         if (!clear) continue;
@@ -96,16 +100,17 @@ __device__ __forceinline__ uint32_t valid_features(const MatchedBank& sb, const 
         } else {
             size = 0.0f;
             for (uint32_t k = sb.off1[ft]; k < sb.off1[ft + 1]; k++)
-                if (w[sb.t1[k].at] > 0.0f) size = __fadd_rn(size, sb.t1[k].v);
+                if (w[sb.t1[k].at] > thr) size = __fadd_rn(size, sb.t1[k].v);
         }
         if (size >= sb.nmin[ft]) valid |= 1u << ft;
     }
     return valid;
 }
 
+// (a tap of weight 0 in one of the three filters adds nothing to its sum)
 __device__ __forceinline__ void sum_features(const MatchedBank& sb, const float* w,
-                                             uint32_t valid, float& E, float& dx, float& dy,
-                                             uint32_t& npix) {
+                                             uint32_t valid, float thr, float& E, float& dx,
+                                             float& dy, uint32_t& npix) {
     E = dx = dy = 0.0f;
     npix = 0;
     bool any = false;
@@ -114,15 +119,19 @@ __device__ __forceinline__ void sum_features(const MatchedBank& sb, const float*
         valid &= valid - 1;
         float drop = 0.0f, mx = 0.0f, my = 0.0f;
         uint32_t under = 0;
-        for (uint32_t k = sb.off1[ft]; k < sb.off1[ft + 1]; k++) {
-            const float sv = w[sb.t1[k].at];
-            drop = __fadd_rn(drop, __fmul_rn(sv, sb.t1[k].v));
-            under += sv > 0.0f;
+        const uint32_t k1 = sb.offs[ft + 1];
+#pragma unroll 4
+        for (uint32_t k = sb.offs[ft]; k < k1; k++) {
+            const MatchedSum t = sb.ts[k];
+            const float e = w[t.at & 0xFFFFu];
+            const float sv = e > thr ? e : 0.0f;
+            if (t.v1 != 0.0f) {
+                drop = __fadd_rn(drop, __fmul_rn(sv, t.v1));
+                under += sv > 0.0f;
+            }
+            if (t.vx != 0.0f) mx = __fadd_rn(mx, __fmul_rn(sv, t.vx));
+            if (t.vy != 0.0f) my = __fadd_rn(my, __fmul_rn(sv, t.vy));
         }
-        for (uint32_t k = sb.offx[ft]; k < sb.offx[ft + 1]; k++)
-            mx = __fadd_rn(mx, __fmul_rn(w[sb.tx[k].at], sb.tx[k].v));
-        for (uint32_t k = sb.offy[ft]; k < sb.offy[ft + 1]; k++)
-            my = __fadd_rn(my, __fmul_rn(w[sb.ty[k].at], sb.ty[k].v));
         if (!any) npix = under;
         any = true;
         E = __fadd_rn(E, drop);
@@ -315,11 +324,11 @@ __global__ void __launch_bounds__(kThreads)
             const int r = r0 + ir, c = c0 + ic;
             if (k < n_cand) {
                 // window tap (i, j) is tile[ir + i][ic + j]
-                const uint32_t valid = valid_features(sb, &tile[ir][ic], win);
+                const uint32_t valid = valid_features(sb, &tile[ir][ic], win, 0.0f);
                 if (valid) {
                     float E, dx, dy;
                     uint32_t npix;
-                    sum_features(sb, &tile[ir][ic], valid, E, dx, dy, npix);
+                    sum_features(sb, &tile[ir][ic], valid, 0.0f, E, dx, dy, npix);
                     if (E != 0.0f)
                         emit = make_hit(p, hhit, E, dx, dy, npix, r, c, frame_base + f, mod_base,
                                         h, n, pix);
@@ -335,20 +344,22 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// Candidates per band tile (a larger count tests every own pixel).
-constexpr uint32_t kMbCap = 3072;
+// Candidates per band tile, and those with a valid feature (a larger count
+// tests every own pixel).
+constexpr uint32_t kMbCap = 2048, kMbValid = 1024;
+
+// Words of a signal bitmap row: 32 real columns each, a zero word on both sides.
+__host__ __device__ inline uint32_t sig_words(uint32_t cols) { return (cols + 31) / 32 + 2; }
 
 // Shared memory of the band kernel for bands of rb rows: the s-tile of
 // rb + 3 rows (one above, two below) at the given pitch, both histograms
 // (plus a spare bin), the candidate list and the list of those with a valid
 // feature, the negated common mode of every (tile row, unit column), the
-// stacked row terms, the candidate bitmap of the own rows and the signal
-// nibbles.
+// stacked row terms and the signal bitmaps of this tile and the next.
 size_t band_smem(const ChainParams& p, uint32_t rb, uint32_t pitch) {
     const size_t nr = rb + 3;
-    return 4 * (nr * pitch + 2 * (size_t)p.hist_bins + 4 + 2 * kMbCap + nr * p.units_per_row +
-                nr + (size_t)(rb + 1) * ((pitch + 31) / 32)) +
-           nr * (pitch / 4);
+    return 4 * (nr * pitch + 2 * (size_t)p.hist_bins + 4 + kMbCap + kMbValid + nr * p.units_per_row +
+                nr + 2 * nr * sig_words(p.cols));
 }
 
 constexpr uint32_t kMaxTaps = PD_MAX_FEATURES * 20;
@@ -363,22 +374,20 @@ __global__ void __launch_bounds__(kBandThreads, 2)
     extern __shared__ __align__(16) uint32_t msm[];
     __shared__ MatchedBank sb;
     __shared__ uint32_t s_nc, s_nv;
-    const uint32_t P = bc.pitch, NQ = P / 4, NR = bc.rb + 3;
+    __shared__ uint32_t s_tap[40];  // candidate test: bitmap word offset << 8 | shift
+    const uint32_t P = bc.pitch, NR = bc.rb + 3;
     float* stile = reinterpret_cast<float*>(msm);  // NR x P; real column c at 4 + c
     uint32_t* hpix = msm + NR * P;                 // hist_bins + spare
     uint32_t* hhit = hpix + p.hist_bins + 4;       // hist_bins
     uint32_t* list = hhit + p.hist_bins;           // kMbCap: row << 16 | column
-    uint32_t* vlist = list + kMbCap;               // kMbCap: list index | valid << 24
-    float* cmt = reinterpret_cast<float*>(vlist + kMbCap);  // NR x units_per_row
+    uint32_t* vlist = list + kMbCap;               // kMbValid: list index | valid << 24
+    float* cmt = reinterpret_cast<float*>(vlist + kMbValid);  // NR x units_per_row
     float* crt = cmt + NR * p.units_per_row;                  // NR row terms
-    // candidate bitmap: bit x of row rl (words of WPR per row, rows 1 ..
-    // rows_here used) marks s-tile column x of own row rl as a pixel whose
-    // window holds signal; zero between tiles
-    const uint32_t WPR = (P + 31) / 32;
-    uint32_t* cbits = reinterpret_cast<uint32_t*>(crt + NR);  // (rb + 1) x WPR
-    // nibble q of a row: signal bits of s-tile columns 4q .. 4q + 3 (real
-    // columns 4q - 4 .. 4q - 1); the first and last nibble stay 0
-    uint8_t* nib = reinterpret_cast<uint8_t*>(cbits + (bc.rb + 1) * WPR);
+    // signal bitmaps of this tile and the next: bit c % 32 of word 1 + c / 32
+    // of a tile row is the signal of real column c
+    const uint32_t W = ((uint32_t)p.cols + 31) / 32, SW = W + 2;
+    uint32_t* sig = reinterpret_cast<uint32_t*>(crt + NR);  // NR x SW, twice
+    uint32_t* sig_next = sig + NR * SW;
 
     const uint32_t tid = threadIdx.x, nthr = blockDim.x;
     const int lane = tid & 31;
@@ -394,8 +403,7 @@ __global__ void __launch_bounds__(kBandThreads, 2)
     const int trash_bits = (int)(kMagicBits + p.hist_bins);
 
     for (uint32_t i = tid; i < NR * P; i += nthr) stile[i] = 0.0f;
-    for (uint32_t i = tid; i < NR * NQ; i += nthr) nib[i] = 0;
-    for (uint32_t i = tid; i < (bc.rb + 1) * WPR; i += nthr) cbits[i] = 0;
+    for (uint32_t i = tid; i < 2 * NR * SW; i += nthr) sig[i] = 0;
     for (uint32_t i = tid; i < 2 * p.hist_bins + 4; i += nthr) hpix[i] = 0;
     {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(bank);
@@ -403,12 +411,30 @@ __global__ void __launch_bounds__(kBandThreads, 2)
         for (uint32_t k = tid; k < sizeof(MatchedBank) / 4; k += nthr) dst[k] = src[k];
     }
     __syncthreads();
+    // the candidate test's taps, those that must be clear first: tap (i, j)
+    // of pixel x is bit x + j - 2 of tile row rl - 1 + i
+    const uint32_t m_clear = sb.clear, m_some = sb.some;
+    const int n_clear = __popc(m_clear), n_test = n_clear + __popc(m_some);
+    if (tid < 40) {
+        const uint32_t k = tid % 20, mask = tid < 20 ? m_clear : m_some;
+        if (mask >> k & 1u) {
+            const int at = (tid < 20 ? 0 : n_clear) + __popc(mask & ((1u << k) - 1u));
+            const uint32_t i = k / 5;
+            const int d = (int)(k % 5) - 2;
+            // (counted from the word before the pixel's, in tile row rl - 1)
+            s_tap[at] = (i * SW + (d < 0 ? 0u : 1u)) << 8 | (uint32_t)(d & 31);
+        }
+    }
     // tap offsets at this pitch
-    for (uint32_t k = tid; k < 4 * kMaxTaps; k += nthr) {
-        MatchedTap* lst = k < kMaxTaps ? sb.t1 : k < 2 * kMaxTaps ? sb.t0
-                                             : k < 3 * kMaxTaps ? sb.tx : sb.ty;
-        MatchedTap& tp = lst[k % kMaxTaps];
-        tp.at = (uint16_t)(tp.i * P + tp.j);
+    for (uint32_t k = tid; k < 3 * kMaxTaps; k += nthr) {
+        if (k < 2 * kMaxTaps) {
+            MatchedTap& tp = k < kMaxTaps ? sb.t1[k] : sb.t0[k - kMaxTaps];
+            tp.at = (uint16_t)(tp.i * P + tp.j);
+        } else {
+            uint32_t& at = sb.ts[k - 2 * kMaxTaps].at;
+            const uint32_t q = at >> 16;
+            at = (q / 5) * P + q % 5;
+        }
     }
 
     // negated common mode of entry i (tile row, unit column) of tile tt; each
@@ -466,119 +492,106 @@ __global__ void __launch_bounds__(kBandThreads, 2)
         if (tid == 0) s_nc = s_nv = 0;
         __syncthreads();
 
-        // 1. zeroed signal and its nibbles of rows r0-1 .. r0+rows_here+1;
-        //    halo rows are not histogrammed (their bins go to the spare bin)
+        // 1. energies and signal bits (zeroed where they are read) of rows r0-1 .. r0+rows_here+1, two
+        //    register sets so that the next row's loads are in flight; halo
+        //    rows are not histogrammed (their bins go to the spare bin)
         if (active) {
             const int nrows = rows_here + 3;
-            constexpr int U = 1;
-            for (int rl0 = (int)ty; rl0 < nrows; rl0 += U * (int)TY) {
-                uint2 rr[U];
-                float4 pp[U], gg[U];
-                bool in[U];
-#pragma unroll
-                for (int j = 0; j < U; j++) {
-                    const int rl = rl0 + j * (int)TY;
-                    const int r = r0 - 1 + rl;
-                    in[j] = rl < nrows && r >= 0 && r < R;
-                    if (in[j]) {
-                        const uint32_t off = (uint32_t)r * p.cols + (uint32_t)col;
-                        rr[j] = *reinterpret_cast<const uint2*>(fr + off);
-                        pp[j] = *reinterpret_cast<const float4*>(npm + off);
-                        gg[j] = *reinterpret_cast<const float4*>(gm + off);
-                    }
+            struct Row {
+                uint2 rw;
+                float4 np, g;
+            };
+            auto inside = [&](int rl) { return r0 - 1 + rl >= 0 && r0 - 1 + rl < R; };
+            auto load = [&](int rl, Row& x) {
+                if (rl >= nrows || !inside(rl)) return;
+                const uint32_t off = (uint32_t)(r0 - 1 + rl) * p.cols + (uint32_t)col;
+                x.rw = __ldg(reinterpret_cast<const uint2*>(fr + off));
+                x.np = __ldg(reinterpret_cast<const float4*>(npm + off));
+                x.g = __ldg(reinterpret_cast<const float4*>(gm + off));
+            };
+            auto row = [&](const Row& x, int rl) {
+                float* srow = stile + rl * P + 4 + col;
+                if (!inside(rl)) {
+                    *reinterpret_cast<float4*>(srow) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    return;
                 }
-#pragma unroll
-                for (int j = 0; j < U; j++) {
-                    const int rl = rl0 + j * (int)TY;
-                    if (rl >= nrows) continue;
-                    float* srow = stile + rl * P + 4 + col;
-                    uint8_t* nq = nib + rl * NQ + tx + 1;
-                    if (!in[j]) {
-                        *reinterpret_cast<float4*>(srow) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                        *nq = 0;
-                        continue;
-                    }
-                    const int r = r0 - 1 + rl;
-                    const bool own = rl >= 1 && rl <= rows_here;
-                    const int blo = own ? (int)kMagicBits : trash_bits;
-                    const int bhi = own ? max_bits : trash_bits;
-                    const float ncma = cmt[rl * p.units_per_row + uca];
-                    const float ncmb = cmt[rl * p.units_per_row + ucb];
-                    const float2 d01 = __fadd2_rn(raw_pair(rr[j].x), make_float2(pp[j].x, pp[j].y));
-                    const float2 d23 = __fadd2_rn(raw_pair(rr[j].y), make_float2(pp[j].z, pp[j].w));
-                    const float2 n01 = make_float2(split > 0 ? ncma : ncmb, split > 1 ? ncma : ncmb);
-                    const float2 n23 = make_float2(split > 2 ? ncma : ncmb, split > 3 ? ncma : ncmb);
-                    float2 c01 = __fadd2_rn(d01, n01), c23 = __fadd2_rn(d23, n23);
-                    if (STACKED) {
-                        const float ncr = crt[rl];
-                        c01 = __fadd2_rn(__fadd2_rn(c01, make_float2(ncr, ncr)),
-                                         make_float2(ncc[0], ncc[1]));
-                        c23 = __fadd2_rn(__fadd2_rn(c23, make_float2(ncr, ncr)),
-                                         make_float2(ncc[2], ncc[3]));
-                    }
-                    const float2 e01 = __fmul2_rn(c01, make_float2(gg[j].x, gg[j].y));
-                    const float2 e23 = __fmul2_rn(c23, make_float2(gg[j].z, gg[j].w));
-                    const float2 iw = make_float2(p.hist_inv_w, p.hist_inv_w);
-                    const float2 nl = make_float2(p.hist_neg_lo_s, p.hist_neg_lo_s);
-                    const float2 mgc = make_float2(kMagic, kMagic);
-                    const float2 u01 = __fadd2_rd(__ffma2_rn(e01, iw, nl), mgc);
-                    const float2 u23 = __fadd2_rd(__ffma2_rn(e23, iw, nl), mgc);
-                    atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u01.x), blo), bhi) - kMagicBits], 1u);
-                    atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u01.y), blo), bhi) - kMagicBits], 1u);
-                    atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u23.x), blo), bhi) - kMagicBits], 1u);
-                    atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u23.y), blo), bhi) - kMagicBits], 1u);
-                    const float e[4] = {e01.x, e01.y, e23.x, e23.y};
-                    float sv[4];
-                    uint32_t bits = 0;
-#pragma unroll
-                    for (int i = 0; i < 4; i++) {
-                        sv[i] = e[i] > p.zero_thr ? e[i] : 0.0f;
-                        bits |= (uint32_t)(sv[i] > 0.0f) << i;
-                    }
-                    *reinterpret_cast<float4*>(srow) = make_float4(sv[0], sv[1], sv[2], sv[3]);
-                    *nq = (uint8_t)bits;
-                    if (bits) {
-                        // signal at row rl, s-tile column x lies in the
-                        // windows of own rows rl-2 .. rl+1, columns x-2 ..
-                        // x+2: an 8-bit run from column col + 2
-                        const uint32_t run = bits | bits << 1 | bits << 2 | bits << 3 | bits << 4;
-                        const uint32_t x0 = (uint32_t)col + 2, w = x0 >> 5, sh = x0 & 31;
-                        const uint32_t lo = run << sh, hi = sh > 24 ? run >> (32 - sh) : 0u;
-                        for (int rr = max(1, rl - 2); rr <= min(rows_here, rl + 1); rr++) {
-                            atomicOr(&cbits[rr * WPR + w], lo);
-                            if (hi) atomicOr(&cbits[rr * WPR + w + 1], hi);
-                        }
-                    }
-                    if (own && out.corrected) {
-                        const uint32_t off = (uint32_t)r * p.cols + (uint32_t)col;
-                        float* dst = out.corrected + (size_t)f * p.frame_px + mod_base + off;
-                        *reinterpret_cast<float4*>(dst) = make_float4(e[0], e[1], e[2], e[3]);
-                    }
+                const bool own = rl >= 1 && rl <= rows_here;
+                const int blo = own ? (int)kMagicBits : trash_bits;
+                const int bhi = own ? max_bits : trash_bits;
+                const float ncma = cmt[rl * p.units_per_row + uca];
+                const float ncmb = cmt[rl * p.units_per_row + ucb];
+                const float2 d01 = __fadd2_rn(raw_pair(x.rw.x), make_float2(x.np.x, x.np.y));
+                const float2 d23 = __fadd2_rn(raw_pair(x.rw.y), make_float2(x.np.z, x.np.w));
+                const float2 n01 = make_float2(split > 0 ? ncma : ncmb, split > 1 ? ncma : ncmb);
+                const float2 n23 = make_float2(split > 2 ? ncma : ncmb, split > 3 ? ncma : ncmb);
+                float2 c01 = __fadd2_rn(d01, n01), c23 = __fadd2_rn(d23, n23);
+                if (STACKED) {
+                    const float ncr = crt[rl];
+                    c01 = __fadd2_rn(__fadd2_rn(c01, make_float2(ncr, ncr)),
+                                     make_float2(ncc[0], ncc[1]));
+                    c23 = __fadd2_rn(__fadd2_rn(c23, make_float2(ncr, ncr)),
+                                     make_float2(ncc[2], ncc[3]));
                 }
+                const float2 e01 = __fmul2_rn(c01, make_float2(x.g.x, x.g.y));
+                const float2 e23 = __fmul2_rn(c23, make_float2(x.g.z, x.g.w));
+                const float2 iw = make_float2(p.hist_inv_w, p.hist_inv_w);
+                const float2 nl = make_float2(p.hist_neg_lo_s, p.hist_neg_lo_s);
+                const float2 mgc = make_float2(kMagic, kMagic);
+                const float2 u01 = __fadd2_rd(__ffma2_rn(e01, iw, nl), mgc);
+                const float2 u23 = __fadd2_rd(__ffma2_rn(e23, iw, nl), mgc);
+                atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u01.x), blo), bhi) - kMagicBits], 1u);
+                atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u01.y), blo), bhi) - kMagicBits], 1u);
+                atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u23.x), blo), bhi) - kMagicBits], 1u);
+                atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u23.y), blo), bhi) - kMagicBits], 1u);
+                const float e[4] = {e01.x, e01.y, e23.x, e23.y};
+                uint32_t bits = 0;
+#pragma unroll
+                for (int i = 0; i < 4; i++) bits |= e[i] > p.zero_thr ? 1u << i : 0u;
+                *reinterpret_cast<float4*>(srow) = make_float4(e[0], e[1], e[2], e[3]);
+                if (bits) atomicOr(&sig[rl * SW + 1 + (col >> 5)], bits << (col & 31));
+                if (own && out.corrected) {
+                    const uint32_t off = (uint32_t)(r0 - 1 + rl) * p.cols + (uint32_t)col;
+                    float* dst = out.corrected + (size_t)f * p.frame_px + mod_base + off;
+                    *reinterpret_cast<float4*>(dst) = make_float4(e[0], e[1], e[2], e[3]);
+                }
+            };
+            Row xa, xb;
+            load((int)ty, xa);
+            for (int rl = (int)ty; rl < nrows; rl += 2 * (int)TY) {
+                load(rl + (int)TY, xb);
+                row(xa, rl);
+                if (rl + (int)TY >= nrows) break;
+                load(rl + 2 * (int)TY, xa);
+                row(xb, rl + (int)TY);
             }
         }
         // the next tile's common mode, in flight during the rest of this one
         if (t + gridDim.x < n_tiles && tid < ncmt) cmv = tile_cm(t + gridDim.x, tid);
         __syncthreads();
 
-        // 2. the marked pixels into a list (a warp scan and one shared
-        //    atomic per warp reserve each thread's slots; list order is
-        //    free), clearing the bitmap for the next tile
-        const uint32_t n_words = (uint32_t)rows_here * WPR;
+        // 2. the candidates into a list (a warp scan and one shared atomic per
+        //    warp reserve each thread's slots; list order is free), the next
+        //    tile's bitmap cleared
+        for (uint32_t i = tid; i < NR * SW; i += nthr) sig_next[i] = 0;
+        const uint32_t n_words = (uint32_t)rows_here * W;
         for (uint32_t base = 0; base < n_words; base += nthr) {
             const uint32_t q = base + tid;
             uint32_t word = 0;
             int rl = 0, x0 = 0;
             if (q < n_words) {
-                rl = 1 + (int)(q / WPR);
-                x0 = 32 * (int)(q % WPR);
-                uint32_t* cw = cbits + rl * WPR + (q % WPR);
-                word = *cw;
-                *cw = 0;
-                // keep s-tile columns 4 .. C + 3 (real columns 0 .. C - 1)
-                if (x0 < 4) word &= 0xFFFFFFFFu << (4 - x0);
-                const int xe = C + 4 - x0;
-                if (xe < 32) word &= xe > 0 ? 0xFFFFFFFFu >> (32 - xe) : 0u;
+                rl = 1 + (int)(q / W);
+                x0 = 32 * (int)(q % W);
+                const uint32_t* s0 = sig + (uint32_t)(rl - 1) * SW + q % W;
+                auto tap = [&](int k) {
+                    const uint32_t t = s_tap[k];
+                    const uint32_t* a = s0 + (t >> 8);
+                    return __funnelshift_r(a[0], a[1], t & 31u);
+                };
+                for (int k = n_clear; k < n_test; k++) word |= tap(k);
+                uint32_t over = 0;
+                for (int k = 0; k < n_clear; k++) over |= tap(k);
+                word &= ~over;
+                if (C - x0 < 32) word &= 0xFFFFFFFFu >> (32 - (C - x0));
             }
             const unsigned wm = __activemask();
             const uint32_t cnt = (uint32_t)__popc(word);
@@ -597,7 +610,7 @@ __global__ void __launch_bounds__(kBandThreads, 2)
             while (word && at < kMbCap) {
                 const int bit = __ffs(word) - 1;
                 word &= word - 1;
-                list[at++] = ((uint32_t)rl << 16) | (uint32_t)(x0 + bit - 4);
+                list[at++] = ((uint32_t)rl << 16) | (uint32_t)(x0 + bit);
             }
         }
         __syncthreads();
@@ -607,11 +620,10 @@ __global__ void __launch_bounds__(kBandThreads, 2)
         //    few with some valid feature (a second list), the sums and the
         //    hit, so that the sums run with every lane on such a pixel
         const uint32_t n_list = s_nc;
-        const bool scan = n_list > kMbCap;
-        const uint32_t n_work = scan ? (uint32_t)rows_here * (uint32_t)C : n_list;
+        bool scan = n_list > kMbCap;
+        uint32_t n_work = scan ? (uint32_t)rows_here * (uint32_t)C : n_list;
         // (row, column) of work item j, and its window mask: rows rl-1 ..
-        // rl+2, columns c-2 .. c+2 are bits 2 + c % 4 .. 6 + c % 4 of
-        // nibbles c / 4 .. c / 4 + 2
+        // rl+2, columns c-2 .. c+2
         auto item_at = [&](uint32_t j, int& rl, int& c) {
             if (scan) {
                 rl = 1 + (int)(j / (uint32_t)C);
@@ -623,15 +635,12 @@ __global__ void __launch_bounds__(kBandThreads, 2)
             }
         };
         auto window = [&](int rl, int c) -> uint32_t {
-            const uint8_t* nw = nib + (rl - 1) * NQ + c / 4;
-            const int sh = 2 + (c & 3);
+            const uint32_t* w = sig + (uint32_t)(rl - 1) * SW + (uint32_t)(c + 30) / 32;
             uint32_t win = 0;
 #pragma unroll
-            for (int i = 0; i < 4; i++) {
-                const uint8_t* g = nw + i * NQ;
-                const uint32_t gr = (uint32_t)g[0] | (uint32_t)g[1] << 4 | (uint32_t)g[2] << 8;
-                win |= ((gr >> sh) & 0x1Fu) << (5 * i);
-            }
+            for (int i = 0; i < 4; i++)
+                win |= (__funnelshift_r(w[i * SW], w[i * SW + 1], (uint32_t)(c + 30) & 31u) & 0x1Fu)
+                       << (5 * i);
             return win;
         };
         if (!scan) {
@@ -642,7 +651,8 @@ __global__ void __launch_bounds__(kBandThreads, 2)
                     int rl, c;
                     item_at(j, rl, c);
                     const uint32_t win = window(rl, c);
-                    if (win) valid = valid_features(sb, stile + (rl - 1) * P + c + 2, win);
+                    if (win) valid = valid_features(sb, stile + (rl - 1) * P + c + 2, win,
+                                                        p.zero_thr);
                 }
                 const unsigned wm = __activemask();
                 const uint32_t bal = __ballot_sync(wm, valid != 0);
@@ -651,10 +661,17 @@ __global__ void __launch_bounds__(kBandThreads, 2)
                     uint32_t at0 = 0;
                     if (lane == lead) at0 = atomicAdd(&s_nv, (uint32_t)__popc(bal));
                     at0 = __shfl_sync(wm, at0, lead);
-                    if (valid) vlist[at0 + __popc(bal & ((1u << lane) - 1u))] = j | valid << 24;
+                    const uint32_t at = at0 + __popc(bal & ((1u << lane) - 1u));
+                    if (valid && at < kMbValid) vlist[at] = j | valid << 24;
                 }
             }
             __syncthreads();
+            if (s_nv > kMbValid) {
+                scan = true;
+                n_work = (uint32_t)rows_here * (uint32_t)C;
+            }
+        }
+        if (!scan) {
             const uint32_t n_valid = s_nv;
             for (uint32_t base = 0; base < n_valid; base += nthr) {
                 const uint32_t k = base + tid;
@@ -667,7 +684,8 @@ __global__ void __launch_bounds__(kBandThreads, 2)
                     item_at(e & 0xFFFFFFu, rl, c);
                     float E, dx, dy;
                     uint32_t npix;
-                    sum_features(sb, stile + (rl - 1) * P + c + 2, e >> 24, E, dx, dy, npix);
+                    sum_features(sb, stile + (rl - 1) * P + c + 2, e >> 24, p.zero_thr, E, dx, dy,
+                                 npix);
                     if (E != 0.0f)
                         emit = make_hit(p, hhit, E, dx, dy, npix, r0 - 1 + rl, c, frame_base + f,
                                         mod_base, h, n, pix);
@@ -685,11 +703,11 @@ __global__ void __launch_bounds__(kBandThreads, 2)
                     item_at(j, rl, c);
                     const uint32_t win = window(rl, c);
                     const float* w = stile + (rl - 1) * P + c + 2;
-                    const uint32_t valid = win ? valid_features(sb, w, win) : 0u;
+                    const uint32_t valid = win ? valid_features(sb, w, win, p.zero_thr) : 0u;
                     if (valid) {
                         float E, dx, dy;
                         uint32_t npix;
-                        sum_features(sb, w, valid, E, dx, dy, npix);
+                        sum_features(sb, w, valid, p.zero_thr, E, dx, dy, npix);
                         if (E != 0.0f)
                             emit = make_hit(p, hhit, E, dx, dy, npix, r0 - 1 + rl, c,
                                             frame_base + f, mod_base, h, n, pix);
@@ -699,6 +717,11 @@ __global__ void __launch_bounds__(kBandThreads, 2)
             }
         }
         __syncthreads();
+        {
+            uint32_t* const other = sig;
+            sig = sig_next;
+            sig_next = other;
+        }
         if (prefetcher && t + 2 * step < n_tiles) {
             TileWalk nx = walk;
             nx.next();
@@ -743,7 +766,7 @@ bool compile_bank(const pd_filter_bank& b, MatchedBank* out) {
     if (b.n_features < 1 || b.n_features > PD_MAX_FEATURES) return false;
     MatchedBank mb{};
     mb.n_features = b.n_features;
-    uint32_t n1 = 0, n0 = 0, nx = 0, ny = 0;
+    uint32_t n1 = 0, n0 = 0, ns = 0;
     for (uint32_t f = 0; f < b.n_features; f++) {
         if (isnan(b.f1_nmin[f])) return false;
         for (int i = 0; i < 4; i++)
@@ -754,8 +777,6 @@ bool compile_bank(const pd_filter_bank& b, MatchedBank* out) {
         mb.nmin[f] = b.f1_nmin[f];
         mb.off1[f] = (uint16_t)n1;
         mb.off0[f] = (uint16_t)n0;
-        mb.offx[f] = (uint16_t)nx;
-        mb.offy[f] = (uint16_t)ny;
         compile_taps(b.f1[f], mb.t1, &n1);
         compile_taps(b.f0[f], mb.t0, &n0);
         mb.f1_unit[f] = mb.f0_pos[f] = 1;
@@ -770,17 +791,26 @@ bool compile_bank(const pd_filter_bank& b, MatchedBank* out) {
                     if (!(b.f0[f][i][j] > 0.0f)) mb.f0_pos[f] = 0;
                 }
             }
-        compile_taps(b.f1_dx[f], mb.tx, &nx);
-        compile_taps(b.f1_dy[f], mb.ty, &ny);
+        mb.offs[f] = (uint16_t)ns;
+        for (int i = 0; i < 4; i++)
+            for (int j = 0; j < 5; j++)
+                if (b.f1[f][i][j] != 0.0f || b.f1_dx[f][i][j] != 0.0f || b.f1_dy[f][i][j] != 0.0f)
+                    mb.ts[ns++] = MatchedSum{(uint32_t)(i * kHX + j) | (uint32_t)(5 * i + j) << 16,
+                                             b.f1[f][i][j], b.f1_dx[f][i][j], b.f1_dy[f][i][j]};
     }
+    mb.offs[b.n_features] = (uint16_t)ns;
     mb.all_binary = 1;
     for (uint32_t f = 0; f < b.n_features; f++)
         if (!mb.f1_unit[f] || !mb.f0_pos[f]) mb.all_binary = 0;
     mb.vtab = nullptr;
+    mb.clear = (1u << 20) - 1u;
+    mb.some = 0;
+    for (uint32_t f = 0; f < b.n_features; f++) {
+        mb.some |= mb.m1[f];
+        mb.clear &= mb.f0_pos[f] ? mb.m0[f] : 0u;
+    }
     mb.off1[b.n_features] = (uint16_t)n1;
     mb.off0[b.n_features] = (uint16_t)n0;
-    mb.offx[b.n_features] = (uint16_t)nx;
-    mb.offy[b.n_features] = (uint16_t)ny;
     *out = mb;
     return true;
 }
@@ -791,6 +821,9 @@ cudaError_t build_vtab(const MatchedBank* bank_dev, uint8_t* vtab) {
     return e != cudaSuccess ? e : cudaDeviceSynchronize();
 }
 
+// dynamic shared memory of one of two CTAs per SM
+constexpr size_t kBandSmem = (size_t)(228 * 1024) / 2 - sizeof(MatchedBank) - 2048;
+
 // Band form of the matched stencil: single gain, raw - pedestal before the
 // common mode, four-pixel chunks (as the band stencil's), and bands of at
 // least one row within about 100 KB of shared memory.
@@ -798,11 +831,16 @@ static bool matched_band_config(const ChainParams& p, BandConfig* out) {
     if (cm_after_gain(p)) return false;
     BandConfig bc = make_band_config(p);
     if (!bc.ok || bc.vec != 4) return false;
-    uint32_t rb = std::min<uint32_t>(std::max<uint32_t>(4, 12288 / p.cols), p.rows);
-    while (rb > 1 && band_smem(p, rb, bc.pitch) > 100 * 1024) rb--;
-    if (band_smem(p, rb, bc.pitch) > 100 * 1024) return false;
-    bc.rb = rb;
-    bc.n_bands = (p.rows + rb - 1) / rb;
+    // the tallest band that two CTAs per SM hold, split evenly over the rows
+    // (the halo is three rows a band)
+    const size_t least = band_smem(p, 0, bc.pitch);
+    if (least >= kBandSmem) return false;
+    const size_t tallest = (kBandSmem - least) / (band_smem(p, 1, bc.pitch) - least);
+    if (tallest == 0) return false;
+    const uint32_t rb = (uint32_t)std::min<size_t>(tallest, p.rows);
+    const uint32_t bands = (p.rows + rb - 1) / rb;
+    bc.rb = (p.rows + bands - 1) / bands;
+    bc.n_bands = (p.rows + bc.rb - 1) / bc.rb;
     *out = bc;
     return true;
 }
@@ -829,7 +867,7 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
         if (g_attr_dev_mband != dev) {
             for (auto k : {matched_band_kernel<false>, matched_band_kernel<true>}) {
                 cudaError_t e = cudaFuncSetAttribute(
-                    k, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+                    k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmem);
                 if (e != cudaSuccess) return e;
             }
             g_attr_dev_mband = dev;

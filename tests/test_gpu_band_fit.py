@@ -34,7 +34,8 @@ def test_small_calls(shape, frames, matched):
     geom, thr = det.geometry(), det.thresholds()
     bank = filters.example_bank() if matched else None
     okw = dict(filters=oracle.filters(**bank)) if matched else {}
-    ref = oracle.process(oracle.geometry(**geom), oracle.thresholds(**thr), ped, gain, raw, **okw)
+    ref = oracle.process(oracle.geometry(**geom), oracle.thresholds(**thr), ped, gain, raw,
+                         want_corrected=True, **okw)
     for band_rows in (0, 5):
         ctx = pd.pd_create(geom, ped, gain, thr)
         if matched:
