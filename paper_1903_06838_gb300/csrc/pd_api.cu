@@ -608,8 +608,6 @@ int create_impl(const pd_geometry* geometry, uint32_t n_gains, uint32_t gain_shi
     }
     p.mean_frac = g.cm_mode >= PD_CM_MEAN && !ag ? pd::mean_frac_bits(p, pedestal_host) : -1;
     cudaError_t e;
-    std::vector<float> nped(fpx);
-    for (size_t i = 0; i < fpx; i++) nped[i] = -pedestal_host[i];
     if ((e = cudaMalloc(&c->d_ped, fpx * 4)) != cudaSuccess ||
         (e = cudaMalloc(&c->d_nped, fpx * 4)) != cudaSuccess ||
         (e = cudaMalloc(&c->d_inv_gain, fpx * 4)) != cudaSuccess ||
@@ -621,12 +619,12 @@ int create_impl(const pd_geometry* geometry, uint32_t n_gains, uint32_t gain_shi
         return fail(PD_ENOMEM, "device allocation failed in pd_create");
     }
     if ((e = cudaMemcpy(c->d_ped, pedestal_host, fpx * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->d_nped, nped.data(), fpx * 4, cudaMemcpyHostToDevice)) ||
+        (e = pd::launch_negate(c->d_ped, c->d_nped, fpx, nullptr)) ||
         (e = cudaMemcpy(c->d_inv_gain, inv.data(), fpx * 4, cudaMemcpyHostToDevice)) ||
         (e = cudaMemset(c->d_count_map, 0, fpx * 4)) ||
         (e = cudaMemset(c->d_hist_pix, 0, p.hist_bins * 8)) ||
         (e = cudaMemset(c->d_hist_hit, 0, p.hist_bins * 8)) ||
-        (e = cudaMemset(c->d_err, 0, 4))) {
+        (e = cudaMemset(c->d_err, 0, 4)) || (e = cudaStreamSynchronize(nullptr))) {
         free_ctx(c);
         return fail_cuda(e, "pd_create upload");
     }

@@ -238,6 +238,19 @@ __global__ void __launch_bounds__(kStThreads)
 
 }  // namespace
 
+// out[i] = -in[i]: the negated pedestals of a new context (uploading them too
+// took as long as the pedestals)
+__global__ void negate_kernel(const float* __restrict__ in, float* __restrict__ out, size_t n) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (size_t)gridDim.x * blockDim.x)
+        out[i] = -in[i];
+}
+
+cudaError_t launch_negate(const float* in, float* out, size_t n, cudaStream_t stream) {
+    negate_kernel<<<device_sm_count(), 512, 0, stream>>>(in, out, n);
+    return cudaGetLastError();
+}
+
 size_t cm_select_smem_bytes(const ChainParams& p) {
     return (size_t)p.unit_px * sizeof(uint32_t);
 }

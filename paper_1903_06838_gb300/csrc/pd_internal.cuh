@@ -173,6 +173,7 @@ int mean_frac_bits(const ChainParams& p, const float* pedestal);
 cudaError_t launch_cm_mean(const ChainParams& p, const uint16_t* raw, uint32_t n_frames,
                            float* cm, cudaStream_t stream);
 
+cudaError_t launch_negate(const float* in, float* out, size_t n, cudaStream_t stream);
 int device_sm_count();
 
 // 5x5 patches of e / photon_kev around hits (pd_net.cu).

@@ -1229,20 +1229,45 @@ bool code_base(const ChainParams& p, const float* pedestal, int n_codes, CodeBas
     const double cut = p.cm_cut;
     const double lo = cut - n_codes / 8.0;
     const size_t fpx = p.frame_px;
-    long long fmin = 0, fmax = 0;
-    float least = INFINITY;  // smallest nonzero |pedestal|
-    out->F.resize(fpx);
+    // smallest nonzero and largest |pedestal| (bits of |x| order like |x|; a
+    // zero's wrap to the top)
+    uint32_t least_bits = ~0u, most_bits = 0;
     for (size_t i = 0; i < fpx; i++) {
-        const float ped = pedestal[i];
-        if (!std::isfinite(ped)) return false;
-        if (ped != 0.0f) least = std::min(least, std::fabs(ped));
-        const long long fv = floor_sum(-8.0 * (double)ped, -8.0 * lo);
-        if (fv < -(1LL << 30) || fv > (1LL << 30)) return false;
-        out->F[i] = (int32_t)fv;
-        fmin = i ? std::min(fmin, fv) : fv;
-        fmax = i ? std::max(fmax, fv) : fv;
+        uint32_t u;
+        memcpy(&u, pedestal + i, 4);
+        u &= 0x7FFFFFFFu;
+        least_bits = std::min(least_bits, u - 1u);
+        most_bits = std::max(most_bits, u);
     }
-    if (std::isfinite(least)) {
+    if (most_bits >= 0x4D000000u) return false;  // 2^27 or more, or not finite
+    long long fmin = 0, fmax = 0;
+    out->F.resize(fpx);
+    int32_t* F = out->F.data();
+    if (std::floor(8.0 * lo) == 8.0 * lo) {
+        // 8 lo a whole number (a cut in eighths): F = floor(-8 ped) - 8 lo,
+        // -8 ped exact in binary32
+        const int32_t off = (int32_t)(-8.0 * lo);
+        int32_t least_f = INT32_MAX, most_f = INT32_MIN;
+        for (size_t i = 0; i < fpx; i++) {
+            const int32_t fv = (int32_t)std::floor(-8.0f * pedestal[i]) + off;
+            F[i] = fv;
+            least_f = std::min(least_f, fv);
+            most_f = std::max(most_f, fv);
+        }
+        fmin = least_f;
+        fmax = most_f;
+    } else {
+        for (size_t i = 0; i < fpx; i++) {
+            const long long fv = floor_sum(-8.0 * (double)pedestal[i], -8.0 * lo);
+            F[i] = (int32_t)fv;
+            fmin = i ? std::min(fmin, fv) : fv;
+            fmax = i ? std::max(fmax, fv) : fv;
+        }
+    }
+    if (least_bits < most_bits) {  // some pedestal is not zero
+        least_bits++;
+        float least;
+        memcpy(&least, &least_bits, 4);
         // d = x - ped is exact in binary32 while |d| < 2^24 ulp-units of ped
         int ex = 0;
         std::frexp((double)least, &ex);  // least in [2^(ex-1), 2^ex)

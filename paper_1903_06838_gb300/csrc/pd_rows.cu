@@ -266,7 +266,9 @@ bool build_row_codes(const ChainParams& p, const float* pedestal, std::vector<ui
     // codes stay below the bit pattern of binary16's infinity
     if (cb.bias + kCodes > 0x7BFF) return false;
     kmap->resize(p.frame_px);
-    for (size_t i = 0; i < p.frame_px; i++) (*kmap)[i] = (uint16_t)(cb.F[i] + cb.bias);
+    const uint32_t bias = (uint32_t)cb.bias;
+    uint16_t* k = kmap->data();
+    for (size_t i = 0; i < p.frame_px; i++) k[i] = (uint16_t)((uint32_t)cb.F[i] + bias);
     *out = RowCodes{nullptr, (uint32_t)cb.rcap, (uint32_t)cb.bias, (uint32_t)(cb.bias + kCodes)};
     return true;
 }
