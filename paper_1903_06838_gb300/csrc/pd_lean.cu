@@ -912,7 +912,7 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const MultiGain&
                             n = (uint32_t)qr;
                         }
                         if (n >= 1) {
-                            const int rl = (int)(at / P), c = (int)(at - (uint32_t)rl * P) - 4;
+                            const int rl = (int)__umulhi(at, lc.pitch_q), c = (int)at - rl * (int)P - 4;
                             const int r = r0 - 1 + rl;
                             if (r == 0 || c == 0 || r == R - 1 || c == C - 1) flags |= PD_HIT_EDGE;
                             pix = (uint32_t)mod_base + (uint32_t)r * p.cols + (uint32_t)c;
@@ -1458,6 +1458,7 @@ LeanConfig make_lean_config(const ChainParams& p, uint32_t rb, bool multigain) {
     lc.tx = p.cols / 4;
     lc.ty = std::max<uint32_t>(1, kLeanThreads / lc.tx);
     lc.pitch = p.cols + 8;
+    lc.pitch_q = (uint32_t)(((1ull << 32) + lc.pitch - 1) / lc.pitch);
     lc.colbank = p.unit_rows == p.rows ? 1u : 0u;
     lc.list_cap = 4096;
     lc.stage_t = 0;  // the band height is chosen without the stage

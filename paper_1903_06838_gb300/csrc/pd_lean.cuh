@@ -83,6 +83,7 @@ struct LeanConfig {
     uint32_t rb;         // rows per band
     uint32_t n_bands;
     uint32_t pitch;      // floats per tile row: 4 zero columns, cols, 4 zero columns
+    uint32_t pitch_q;    // ceil(2^32 / pitch): a tile offset below 2^16 divided by it
     uint32_t colbank;    // 1: units span the module's full height
     uint32_t list_cap;   // seed candidates per tile
     uint32_t ctas_per_sm;  // persistent CTAs per SM of a launch (0: as shared memory allows)
