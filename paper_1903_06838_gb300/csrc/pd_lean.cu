@@ -709,12 +709,25 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const MultiGain&
                 // common mode, 0 past the last stage
                 const uint32_t hi = 0x10001u * (0xFFFFu & ~mg.vmask);
                 if ((x.rw.x | x.rw.y) & hi) {
+                    // (the four pixels' maps are loaded together: bright spots
+                    // fill whole chunks, and one by one they were four waits: 64
+                    // frames of 32 x 185 x 388, the call 734 -> 721 us)
                     const size_t px = mod_base + (size_t)(r0 - 1 + rl) * p.cols + col;
+                    uint32_t w[4], st[4];
+                    float mp[4], mi[4];
 #pragma unroll
                     for (int i = 0; i < 4; i++) {
-                        const uint32_t w = ((i < 2 ? x.rw.x : x.rw.y) >> (16 * (i & 1))) & 0xFFFFu;
-                        if (w >> mg.shift) {
-                            const float e = mg_energy(mg, p.frame_px, (uint16_t)w, px + i, 0.0f);
+                        w[i] = ((i < 2 ? x.rw.x : x.rw.y) >> (16 * (i & 1))) & 0xFFFFu;
+                        st[i] = w[i] >> mg.shift;
+                        const size_t at = (size_t)(st[i] < mg.n_gains ? st[i] : 0u) * p.frame_px + px + i;
+                        mp[i] = __ldg(mg.ped + at);
+                        mi[i] = __ldg(mg.inv_gain + at);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const float d = __fsub_rn(__uint2float_rn(w[i] & mg.vmask), mp[i]);
+                        const float e = st[i] < mg.n_gains ? __fmul_rn(d, mi[i]) : 0.0f;
+                        if (st[i]) {
                             if (i == 0) e01.x = e;
                             if (i == 1) e01.y = e;
                             if (i == 2) e23.x = e;
