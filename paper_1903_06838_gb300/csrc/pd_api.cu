@@ -258,34 +258,43 @@ bool fused_on(const pd_ctx* c) { return c->use_fused && !c->two_pass && !c->matc
 // (use_fused and use_cm_rows are off for multi-gain contexts: those
 // kernels read single-gain words)
 
-// The charge-summing launch of a context (after its common mode).
+// The charge-summing launch of a context (after its common mode; early: that
+// was the launch before in the stream, and this one may start as it ends).
 cudaError_t launch_stencil_for(const pd_ctx* c, const uint16_t* fr, uint32_t nf,
-                               uint32_t frame_base, const pd::CallOut& co, cudaStream_t s) {
+                               uint32_t frame_base, const pd::CallOut& co, cudaStream_t s,
+                               bool early) {
     const pd::MultiGain* mg = c->multigain ? &c->mg : nullptr;
     if (c->matched)
         return pd::launch_matched(c->params, c->d_bank, fr, nf, frame_base, co, s, mg);
     if (c->use_lean && c->kernels == 1) {
         pd::LeanConfig lc = c->lean_cfg;
         lc.wait_polls = c->wait_polls;
-        return pd::launch_stencil_lean(c->params, lc, fr, nf, frame_base, co, c->d_err, s, mg);
+        return pd::launch_stencil_lean(c->params, lc, fr, nf, frame_base, co, c->d_err, s, mg, early);
     }
     return c->use_band || c->use_band_ag
                ? pd::launch_stencil_band(c->params, c->band_cfg, fr, nf, frame_base, co, s, mg)
                : pd::launch_stencil(c->params, fr, nf, frame_base, co, s, mg);
 }
 
-// The common-mode launch(es) of a context for nf frames into cm.
+// The common-mode launch clears the hit counter of its call.
+bool cm_clears(const pd_ctx* c) {
+    return pd::cm_kind(c->params) == PD_CM_MEDIAN && (c->use_bank || c->use_row_codes) &&
+           c->kernels == 1;
+}
+
+// The common-mode launch(es) of a context for nf frames into cm; zero: a word
+// to clear (cm_clears), or NULL.
 cudaError_t launch_cm(const pd_ctx* c, const uint16_t* fr, uint32_t nf, float* cm,
-                      cudaStream_t s) {
+                      cudaStream_t s, uint32_t* zero = nullptr) {
     if (pd::cm_kind(c->params) == PD_CM_MEAN || pd::cm_kind(c->params) == PD_CM_MEAN_STACKED)
         return pd::launch_cm_mean(c->params, fr, nf, cm, s);
     if (c->use_bank && c->kernels == 1) {
         pd::CodeMap cmap = c->cmap;
         cmap.wait_polls = c->wait_polls;
-        return pd::launch_cm_bank(c->params, c->cm_cfg, cmap, fr, nf, cm, c->d_err, s);
+        return pd::launch_cm_bank(c->params, c->cm_cfg, cmap, fr, nf, cm, c->d_err, s, zero);
     }
     if (c->use_row_codes && c->kernels == 1)
-        return pd::launch_row_codes(c->params, c->row_codes, fr, nf, cm, s);
+        return pd::launch_row_codes(c->params, c->row_codes, fr, nf, cm, s, zero);
     if (c->multigain)
         return c->use_cm_big ? pd::launch_cm_big(c->params, c->cm_cfg, fr, nf, cm, s,
                                                  ~c->mg.vmask & 0xFFFFu)
@@ -335,7 +344,11 @@ int ensure_qsync(pd_ctx* c, uint32_t n_frames) {
 int run_chain(pd_ctx* c, const uint16_t* frames, uint32_t n_frames, uint32_t frame_base,
               const pd_outputs* out, cudaStream_t s, bool zero = true) {
     cudaError_t e = cudaSuccess;
-    if (zero && (e = cudaMemsetAsync(out->n_hits, 0, sizeof(uint32_t), s)) != cudaSuccess)
+    // one launch less where the common mode clears the counter
+    uint32_t* clear = zero && n_frames && !fused_on(c) && !queue_on(c, out) && cm_clears(c)
+                          ? out->n_hits : nullptr;
+    if (zero && !clear &&
+        (e = cudaMemsetAsync(out->n_hits, 0, sizeof(uint32_t), s)) != cudaSuccess)
         return fail_cuda(e, "zero n_hits");
     if (n_frames == 0) return PD_OK;
     if (fused_on(c)) {
@@ -384,7 +397,7 @@ int run_chain(pd_ctx* c, const uint16_t* frames, uint32_t n_frames, uint32_t fra
             return fail_cuda(e, "chunk pipeline wait");
         {
             ProfileScope ps(c, 0, sc);
-            e = launch_cm(c, fr, nf, cmc, sc);
+            e = launch_cm(c, fr, nf, cmc, sc, done ? nullptr : clear);
         }
         if (e != cudaSuccess) return fail_cuda(e, "common-mode kernel launch");
         if (two && ((e = cudaEventRecord(c->ev_cm[k & 1], sc)) ||
@@ -396,7 +409,7 @@ int run_chain(pd_ctx* c, const uint16_t* frames, uint32_t n_frames, uint32_t fra
                        cmc};
         {
             ProfileScope ps(c, 1, s);
-            e = launch_stencil_for(c, fr, nf, frame_base + done, co, s);
+            e = launch_stencil_for(c, fr, nf, frame_base + done, co, s, !two && !c->profiling);
         }
         if (e != cudaSuccess) return fail_cuda(e, "stencil kernel launch");
         if (two && (e = cudaEventRecord(c->ev_st[k & 1], s)))
@@ -460,7 +473,7 @@ int internal_run_sequential(pd_ctx* c, const uint16_t* frames, uint32_t n_frames
                    out->corrected ? out->corrected + (size_t)done * c->params.frame_px
                                   : nullptr,
                    cmc};
-        e = launch_stencil_for(c, fr, nf, frame_base + done, co, s);
+        e = launch_stencil_for(c, fr, nf, frame_base + done, co, s, true);
         if (e != cudaSuccess) return fail_cuda(e, "stencil kernel launch");
         done += nf;
     }

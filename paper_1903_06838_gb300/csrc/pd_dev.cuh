@@ -112,6 +112,16 @@ __device__ __forceinline__ uint32_t cm_code(float d, float magic_w) {
     return (uint32_t)(b - (int)kMagicBits);
 }
 
+// Programmatic dependent launch: the kernel before this one in the stream is
+// complete and its writes are visible (at once where it was launched without);
+// the next one may start once every CTA has said so or is done.
+__device__ __forceinline__ void wait_previous_kernel() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void start_next_kernel() {
+    asm volatile("griddepcontrol.launch_dependents;");
+}
+
 // Asynchronous 4-byte global -> shared copy (no register staging), and the
 // wait for all of this thread's copies.
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {

@@ -479,8 +479,10 @@ __device__ __forceinline__ bool cm_bank_item(const ChainParams& p, float* __rest
 __global__ void __launch_bounds__(kBankThreads, 2)
     cm_bank_kernel(ChainParams p, float* __restrict__ cm_out, CmBigConfig cfg, CodeMap cmap,
                    const __grid_constant__ CUtensorMap frames, const uint16_t* __restrict__ raw,
-                   uint32_t n_items, uint32_t* __restrict__ err) {
+                   uint32_t n_items, uint32_t* __restrict__ err, uint32_t* __restrict__ zero) {
     extern __shared__ __align__(128) uint4 stage[];  // t * ne_box groups of 8 words
+    start_next_kernel();
+    if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
     __shared__ BankShared sh;
     const uint32_t ne = cmap.t * cmap.ne_box;
     BankSmem sm;
@@ -1017,6 +1019,8 @@ __global__ void __launch_bounds__(kLeanThreads, 2)
     __syncthreads();
 
     const LeanLane lane = lean_lane(p, lc);
+    // the common mode (this kernel may start while it ends, launch_stencil_lean)
+    wait_previous_kernel();
     const unsigned long long first = blockIdx.x, step = gridDim.x;
     TileWalk walk(first, step, lc.n_bands, p.n_modules);
     // unstaged: the last thread (a halo lane, which owns the fewest rows)
@@ -1418,7 +1422,7 @@ static cudaError_t encode_bank_map(const ChainParams& p, const CodeMap& cmap,
 
 cudaError_t launch_cm_bank(const ChainParams& p, const CmBigConfig& cfg, const CodeMap& cmap,
                            const uint16_t* raw, uint32_t n_frames, float* cm, uint32_t* err,
-                           cudaStream_t stream) {
+                           cudaStream_t stream, uint32_t* zero) {
     const unsigned long long items = (unsigned long long)n_frames * p.units_per_frame;
     if (items == 0) return cudaSuccess;
     int dev = 0;
@@ -1440,7 +1444,7 @@ cudaError_t launch_cm_bank(const ChainParams& p, const CmBigConfig& cfg, const C
     const unsigned long long grid = std::min<unsigned long long>(
         items, (unsigned long long)std::max<uint32_t>(cmap.ctas_per_sm, 1) * device_sm_count());
     cm_bank_kernel<<<(unsigned)grid, kBankThreads, smem, stream>>>(p, cm, cfg, cmap, map, raw,
-                                                                   (uint32_t)items, err);
+                                                                   (uint32_t)items, err, zero);
     return cudaGetLastError();
 }
 
@@ -1558,7 +1562,7 @@ auto lean_pick(bool colbank, bool oneunit) {
 
 cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& cfg, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
-                                uint32_t* err, cudaStream_t stream, const MultiGain* mg) {
+                                uint32_t* err, cudaStream_t stream, const MultiGain* mg, bool early) {
     if (n_frames == 0) return cudaSuccess;
     LeanConfig lc = cfg;
     if (lc.fit) {
@@ -1631,9 +1635,23 @@ cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& cfg, con
     else if (cm_kind(p) == PD_CM_MEAN_STACKED)
         k = corr ? lean_pick_extra<true, kStacked>(lc.colbank)
                  : lean_pick_extra<false, kStacked>(lc.colbank);
-    k<<<(unsigned)grid, threads, smem, stream>>>(p, raw, frame_base, out, lc, n_tiles, map, err,
-                                                 mg ? *mg : MultiGain{});
-    return cudaGetLastError();
+    // early: the common mode's kernel is the one before in the stream.  This
+    // one may start when all of its CTAs have, clear its shared memory beside
+    // them, and wait for their end before it reads their values.  With the
+    // counter cleared by the common mode (one launch less), a 704 x 768 frame
+    // with its corrected energies: 14.5 -> 11.5 us a call.
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg_l{};
+    cfg_l.gridDim = dim3((unsigned)grid);
+    cfg_l.blockDim = dim3(threads);
+    cfg_l.dynamicSmemBytes = smem;
+    cfg_l.stream = stream;
+    cfg_l.attrs = &attr;
+    cfg_l.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg_l, k, p, raw, frame_base, out, (const LeanConfig)lc, n_tiles,
+                              (const CUtensorMap)map, err, mg ? *mg : MultiGain{});
 }
 
 // ---------------------------------------------------------------------------

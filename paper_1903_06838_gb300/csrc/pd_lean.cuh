@@ -60,7 +60,8 @@ struct RowCodes {
 bool build_row_codes(const ChainParams& p, const float* pedestal, std::vector<uint16_t>* kmap,
                      RowCodes* out);
 cudaError_t launch_row_codes(const ChainParams& p, const RowCodes& rc, const uint16_t* raw,
-                             uint32_t n_frames, float* cm, cudaStream_t stream);
+                             uint32_t n_frames, float* cm, cudaStream_t stream,
+                             uint32_t* zero = nullptr);
 
 // Host side: the map of a geometry and pedestal (out->kmap left null), or
 // false when the integer codes are not exact, do not fit 16-bit lanes, or the
@@ -72,10 +73,11 @@ bool build_code_map(const ChainParams& p, const float* pedestal, std::vector<uin
 size_t cm_bank_smem_bytes(const ChainParams& p, const CodeMap& cmap);
 bool cm_bank_supported(const ChainParams& p, const CodeMap& cmap);
 // err: context error word (bit 0: a bounded wait for the staged copies gave
-// up).  raw: 16-byte aligned frames of frame_px % 8 == 0 words.
+// up).  raw: 16-byte aligned frames of frame_px % 8 == 0 words.  zero: a word
+// the launch clears (the call's hit counter), or NULL; so in launch_row_codes.
 cudaError_t launch_cm_bank(const ChainParams& p, const CmBigConfig& cfg, const CodeMap& cmap,
                            const uint16_t* raw, uint32_t n_frames, float* cm, uint32_t* err,
-                           cudaStream_t stream);
+                           cudaStream_t stream, uint32_t* zero = nullptr);
 
 // Lean stencil over bands of full-width rows (four-pixel chunks).
 struct LeanConfig {
@@ -102,11 +104,12 @@ struct LeanConfig {
 LeanConfig make_lean_config(const ChainParams& p, uint32_t rb = 0, bool multigain = false);
 size_t lean_smem_bytes(const ChainParams& p, const LeanConfig& lc);
 // raw: 16-byte aligned.  err: context error word (bit 1: a bounded wait
-// for a staged copy gave up).  mg: auto-ranging words, or NULL.
+// for a staged copy gave up).  mg: auto-ranging words, or NULL.  early: the
+// launch before in the stream is this call's common mode.
 cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& lc, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
                                 uint32_t* err, cudaStream_t stream,
-                                const MultiGain* mg = nullptr);
+                                const MultiGain* mg = nullptr, bool early = false);
 
 // The lean pair as one persistent launch over a work queue (bank items of
 // frames [sK, sK + K) then the stencil tiles of the K frames before them, K

@@ -116,8 +116,10 @@ __global__ void __launch_bounds__(32 * kRowUnitWarps, 5)
     cm_row_codes_kernel(RowCodes rc, const uint16_t* __restrict__ raw,
                         const float* __restrict__ nped, float* __restrict__ cm,
                         uint32_t n_items, uint32_t units_per_frame, uint32_t npx,
-                        uint32_t min_count, float cut) {
+                        uint32_t min_count, float cut, uint32_t* __restrict__ zero) {
     constexpr int W = 2 * NC;
+    start_next_kernel();
+    if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
     __shared__ RowShared shared[kRowUnitWarps];
     RowShared& S = shared[threadIdx.x >> 5];
     const uint32_t lane = threadIdx.x & 31;
@@ -274,7 +276,7 @@ bool build_row_codes(const ChainParams& p, const float* pedestal, std::vector<ui
 }
 
 cudaError_t launch_row_codes(const ChainParams& p, const RowCodes& rc, const uint16_t* raw,
-                             uint32_t n_frames, float* cm, cudaStream_t stream) {
+                             uint32_t n_frames, float* cm, cudaStream_t stream, uint32_t* zero) {
     // (items indexed in 32 bits: frames in groups)
     const uint32_t group = std::max(1u, (1u << 30) / p.units_per_frame);
     for (uint32_t f0 = 0; f0 < n_frames; f0 += group) {
@@ -288,7 +290,7 @@ cudaError_t launch_row_codes(const ChainParams& p, const RowCodes& rc, const uin
                            : cm_row_codes_kernel<4>;
         k<<<grid, 32 * kRowUnitWarps, 0, stream>>>(
             rc, raw + (size_t)f0 * p.frame_px, p.nped, cm + (size_t)f0 * p.units_per_frame, items,
-            p.units_per_frame, p.unit_px, p.cm_min_count, p.cm_cut);
+            p.units_per_frame, p.unit_px, p.cm_min_count, p.cm_cut, f0 ? nullptr : zero);
     }
     return cudaGetLastError();
 }
