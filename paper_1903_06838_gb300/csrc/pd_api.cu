@@ -265,14 +265,14 @@ cudaError_t launch_stencil_for(const pd_ctx* c, const uint16_t* fr, uint32_t nf,
                                bool early) {
     const pd::MultiGain* mg = c->multigain ? &c->mg : nullptr;
     if (c->matched)
-        return pd::launch_matched(c->params, c->d_bank, fr, nf, frame_base, co, s, mg);
+        return pd::launch_matched(c->params, c->d_bank, fr, nf, frame_base, co, s, mg, early);
     if (c->use_lean && c->kernels == 1) {
         pd::LeanConfig lc = c->lean_cfg;
         lc.wait_polls = c->wait_polls;
         return pd::launch_stencil_lean(c->params, lc, fr, nf, frame_base, co, c->d_err, s, mg, early);
     }
     return c->use_band || c->use_band_ag
-               ? pd::launch_stencil_band(c->params, c->band_cfg, fr, nf, frame_base, co, s, mg)
+               ? pd::launch_stencil_band(c->params, c->band_cfg, fr, nf, frame_base, co, s, mg, early)
                : pd::launch_stencil(c->params, fr, nf, frame_base, co, s, mg);
 }
 

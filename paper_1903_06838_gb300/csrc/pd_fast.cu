@@ -653,6 +653,8 @@ __device__ void stencil_band_run(const ChainParams& p, const uint16_t* __restric
         return -out.cm[fbase + ((uint32_t)r / p.unit_rows) * p.units_per_row +
                        i % p.units_per_row];
     };
+    // the common mode (this kernel may start while it ends, launch_stencil_band)
+    if (PREFETCH) wait_previous_kernel();
     float cmv = 0.0f;
     if (first < n_tiles && tid < ncmt) cmv = tile_cm((uint32_t)first, tid);
 
@@ -1246,7 +1248,7 @@ size_t band_smem_bytes(const ChainParams& p, uint32_t rb, uint32_t pitch) {
 
 cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& cfg, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
-                                cudaStream_t stream, const MultiGain* mg) {
+                                cudaStream_t stream, const MultiGain* mg, bool early) {
     if (n_frames == 0) return cudaSuccess;
     BandConfig bc = cfg;
     const auto ctas_per_sm = [&] {
@@ -1292,8 +1294,19 @@ cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& cfg, con
                               : stencil_band_kernel<4, false, false, true>)
                         : (st ? stencil_band_kernel<1, true, false, true>
                               : stencil_band_kernel<1, false, false, true>);
-    k<<<(unsigned)grid, threads, smem, stream>>>(p, raw, frame_base, out, bc, n_tiles, m);
-    return cudaGetLastError();
+    // (early: as in launch_stencil_lean)
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3((unsigned)grid);
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    lc.attrs = &attr;
+    lc.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, k, p, raw, frame_base, out, (const BandConfig)bc, n_tiles,
+                              (const MultiGain)m);
 }
 
 }  // namespace pd

@@ -111,10 +111,12 @@ cudaError_t launch_cm_rows(const ChainParams& p, const uint16_t* raw, uint32_t n
 BandConfig make_band_config(const ChainParams& p);
 size_t band_smem_bytes(const ChainParams& p, uint32_t rb, uint32_t pitch);
 // mg: auto-ranging words (four-pixel chunks and the median or no common
-// mode only), or NULL.
+// mode only), or NULL.  early: the launch before in the stream is this call's
+// common mode.
 cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& bc, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
-                                cudaStream_t stream, const MultiGain* mg = nullptr);
+                                cudaStream_t stream, const MultiGain* mg = nullptr,
+                                bool early = false);
 
 // Whole chain in one persistent kernel per (frame, module) for modules whose
 // common-mode units are full-height column banks (at most kFusedMaxUnits per

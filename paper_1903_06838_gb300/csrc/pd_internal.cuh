@@ -167,7 +167,7 @@ cudaError_t build_vtab(const MatchedBank* bank_dev, uint8_t* vtab);
 cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
                            const uint16_t* raw, uint32_t n_frames, uint32_t frame_base,
                            const CallOut& out, cudaStream_t stream,
-                           const MultiGain* mg = nullptr);
+                           const MultiGain* mg = nullptr, bool early = false);
 // The paper's mean estimator, one stage or three stacked (pd_cm_mean.cu).
 int mean_frac_bits(const ChainParams& p, const float* pedestal);
 cudaError_t launch_cm_mean(const ChainParams& p, const uint16_t* raw, uint32_t n_frames,

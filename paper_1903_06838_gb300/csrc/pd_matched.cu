@@ -365,8 +365,10 @@ size_t band_smem(const ChainParams& p, uint32_t rb, uint32_t pitch) {
 constexpr uint32_t kMaxTaps = PD_MAX_FEATURES * 20;
 
 // Bands of rb rows of (frame, module): tile t is band t % n_bands of module
-// (t / n_bands) % n_modules of frame t / (n_bands * n_modules).
-template <bool STACKED>
+// (t / n_bands) % n_modules of frame t / (n_bands * n_modules).  COLBANK: the
+// common-mode units span the module's full height, so a thread's four pixels
+// take the same two values on every row of a tile, held in registers.
+template <bool STACKED, bool COLBANK>
 __global__ void __launch_bounds__(kBandThreads, 2)
     matched_band_kernel(ChainParams p, const MatchedBank* __restrict__ bank,
                         const uint16_t* __restrict__ raw, uint32_t frame_base, CallOut out,
@@ -400,7 +402,6 @@ __global__ void __launch_bounds__(kBandThreads, 2)
     const uint32_t ucb = (uint32_t)(col + 3) / p.unit_cols;
     const int split = (int)(ucb * p.unit_cols) - col;  // pixels i >= split use ucb
     const int max_bits = (int)(kMagicBits + p.hist_bins - 1);
-    const int trash_bits = (int)(kMagicBits + p.hist_bins);
 
     for (uint32_t i = tid; i < NR * P; i += nthr) stile[i] = 0.0f;
     for (uint32_t i = tid; i < 2 * NR * SW; i += nthr) sig[i] = 0;
@@ -451,10 +452,23 @@ __global__ void __launch_bounds__(kBandThreads, 2)
         return -out.cm[fbase + ((uint32_t)r / p.unit_rows) * p.units_per_row +
                        i % p.units_per_row];
     };
-    float cmv = 0.0f;
-    if (blockIdx.x < n_tiles && tid < ncmt) cmv = tile_cm(blockIdx.x, tid);
-
+    // (COLBANK: the two values of this thread's chunk)
+    auto chunk_cm = [&](const TileWalk& w) {
+        const float* cmf = out.cm +
+                           (size_t)w.f * (STACKED ? cm_per_frame(p) : p.units_per_frame) +
+                           (size_t)w.m * p.units_per_module;
+        return make_float2(-__ldcg(cmf + uca), -__ldcg(cmf + ucb));
+    };
+    // the common mode (this kernel may start while it ends, launch_matched)
+    wait_previous_kernel();
     TileWalk walk(blockIdx.x, gridDim.x, bc.n_bands, p.n_modules);
+    float cmv = 0.0f;
+    float2 cm2 = make_float2(0.0f, 0.0f);
+    if (COLBANK && active)
+        cm2 = chunk_cm(walk);
+    else if (!COLBANK && blockIdx.x < n_tiles && tid < ncmt)
+        cmv = tile_cm(blockIdx.x, tid);
+
     // the last thread asks L2 for the raw rows (the halo row above, two
     // below) of the next tile now and of the tile after next once a tile is
     // done, so that their loads find them there
@@ -475,8 +489,12 @@ __global__ void __launch_bounds__(kBandThreads, 2)
         const float* npm = p.nped + mod_base;
         const float* gm = p.inv_gain + mod_base;
 
-        if (tid < ncmt) cmt[tid] = cmv;
-        for (uint32_t i = tid + nthr; i < ncmt; i += nthr) cmt[i] = tile_cm(t, i);
+        if (!COLBANK) {
+            if (tid < ncmt) cmt[tid] = cmv;
+            for (uint32_t i = tid + nthr; i < ncmt; i += nthr) cmt[i] = tile_cm(t, i);
+        }
+        const float2 b01 = make_float2(split > 0 ? cm2.x : cm2.y, split > 1 ? cm2.x : cm2.y);
+        const float2 b23 = make_float2(split > 2 ? cm2.x : cm2.y, split > 3 ? cm2.x : cm2.y);
         float ncc[4];
         if (STACKED) {
             const float* cmf = out.cm + (size_t)f * cm_per_frame(p) + p.units_per_frame;
@@ -494,7 +512,7 @@ __global__ void __launch_bounds__(kBandThreads, 2)
 
         // 1. energies and signal bits (zeroed where they are read) of rows r0-1 .. r0+rows_here+1, two
         //    register sets so that the next row's loads are in flight; halo
-        //    rows are not histogrammed (their bins go to the spare bin)
+        //    rows are not histogrammed
         if (active) {
             const int nrows = rows_here + 3;
             struct Row {
@@ -516,14 +534,15 @@ __global__ void __launch_bounds__(kBandThreads, 2)
                     return;
                 }
                 const bool own = rl >= 1 && rl <= rows_here;
-                const int blo = own ? (int)kMagicBits : trash_bits;
-                const int bhi = own ? max_bits : trash_bits;
-                const float ncma = cmt[rl * p.units_per_row + uca];
-                const float ncmb = cmt[rl * p.units_per_row + ucb];
                 const float2 d01 = __fadd2_rn(raw_pair(x.rw.x), make_float2(x.np.x, x.np.y));
                 const float2 d23 = __fadd2_rn(raw_pair(x.rw.y), make_float2(x.np.z, x.np.w));
-                const float2 n01 = make_float2(split > 0 ? ncma : ncmb, split > 1 ? ncma : ncmb);
-                const float2 n23 = make_float2(split > 2 ? ncma : ncmb, split > 3 ? ncma : ncmb);
+                float2 n01 = b01, n23 = b23;
+                if (!COLBANK) {
+                    const float ncma = cmt[rl * p.units_per_row + uca];
+                    const float ncmb = cmt[rl * p.units_per_row + ucb];
+                    n01 = make_float2(split > 0 ? ncma : ncmb, split > 1 ? ncma : ncmb);
+                    n23 = make_float2(split > 2 ? ncma : ncmb, split > 3 ? ncma : ncmb);
+                }
                 float2 c01 = __fadd2_rn(d01, n01), c23 = __fadd2_rn(d23, n23);
                 if (STACKED) {
                     const float ncr = crt[rl];
@@ -539,10 +558,16 @@ __global__ void __launch_bounds__(kBandThreads, 2)
                 const float2 mgc = make_float2(kMagic, kMagic);
                 const float2 u01 = __fadd2_rd(__ffma2_rn(e01, iw, nl), mgc);
                 const float2 u23 = __fadd2_rd(__ffma2_rn(e23, iw, nl), mgc);
-                atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u01.x), blo), bhi) - kMagicBits], 1u);
-                atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u01.y), blo), bhi) - kMagicBits], 1u);
-                atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u23.x), blo), bhi) - kMagicBits], 1u);
-                atomicAdd(&hpix[(uint32_t)min(max(__float_as_int(u23.y), blo), bhi) - kMagicBits], 1u);
+                if (own) {
+                    auto count = [&](float u) {
+                        const int b = min(max(__float_as_int(u), (int)kMagicBits), max_bits);
+                        atomicAdd(&hpix[(uint32_t)b - kMagicBits], 1u);
+                    };
+                    count(u01.x);
+                    count(u01.y);
+                    count(u23.x);
+                    count(u23.y);
+                }
                 const float e[4] = {e01.x, e01.y, e23.x, e23.y};
                 uint32_t bits = 0;
 #pragma unroll
@@ -566,7 +591,15 @@ __global__ void __launch_bounds__(kBandThreads, 2)
             }
         }
         // the next tile's common mode, in flight during the rest of this one
-        if (t + gridDim.x < n_tiles && tid < ncmt) cmv = tile_cm(t + gridDim.x, tid);
+        if (t + gridDim.x < n_tiles) {
+            if (COLBANK && active) {
+                TileWalk nx = walk;
+                nx.next();
+                cm2 = chunk_cm(nx);
+            } else if (!COLBANK && tid < ncmt) {
+                cmv = tile_cm(t + gridDim.x, tid);
+            }
+        }
         __syncthreads();
 
         // 2. the candidates into a list (a warp scan and one shared atomic per
@@ -849,7 +882,8 @@ static int g_attr_dev_mband = -1;
 
 cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
                            const uint16_t* raw, uint32_t n_frames, uint32_t frame_base,
-                           const CallOut& out, cudaStream_t stream, const MultiGain* mg) {
+                           const CallOut& out, cudaStream_t stream, const MultiGain* mg,
+                           bool early) {
     BandConfig bc;
     if (!mg && matched_band_config(p, &bc)) {
         if (n_frames == 0) return cudaSuccess;
@@ -865,7 +899,8 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
         int dev = 0;
         cudaGetDevice(&dev);
         if (g_attr_dev_mband != dev) {
-            for (auto k : {matched_band_kernel<false>, matched_band_kernel<true>}) {
+            for (auto k : {matched_band_kernel<false, false>, matched_band_kernel<false, true>,
+                           matched_band_kernel<true, false>, matched_band_kernel<true, true>}) {
                 cudaError_t e = cudaFuncSetAttribute(
                     k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmem);
                 if (e != cudaSuccess) return e;
@@ -876,13 +911,22 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
         unsigned long long grid = (unsigned long long)device_sm_count() * ctas_per_sm();
         if (grid > n_tiles) grid = n_tiles;
         const unsigned threads = bc.tx * bc.ty;
-        if (cm_kind(p) == PD_CM_MEAN_STACKED)
-            matched_band_kernel<true><<<(unsigned)grid, threads, smem, stream>>>(
-                p, bank_dev, raw, frame_base, out, bc, n_tiles);
-        else
-            matched_band_kernel<false><<<(unsigned)grid, threads, smem, stream>>>(
-                p, bank_dev, raw, frame_base, out, bc, n_tiles);
-        return cudaGetLastError();
+        const bool st = cm_kind(p) == PD_CM_MEAN_STACKED, col = p.unit_rows == p.rows;
+        auto k = st ? (col ? matched_band_kernel<true, true> : matched_band_kernel<true, false>)
+                    : (col ? matched_band_kernel<false, true> : matched_band_kernel<false, false>);
+        // (early: as in launch_stencil_lean)
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cfg.attrs = &attr;
+        cfg.numAttrs = early ? 1 : 0;
+        return cudaLaunchKernelEx(&cfg, k, p, bank_dev, raw, frame_base, out, (const BandConfig)bc,
+                                  n_tiles);
     }
     const uint32_t tiles_y = (p.rows + kTY - 1) / kTY;
     const uint32_t tiles_x = (p.cols + kTX - 1) / kTX;
