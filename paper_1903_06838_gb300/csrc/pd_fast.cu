@@ -1233,6 +1233,11 @@ BandConfig make_band_config(const ChainParams& p) {
     rb = std::min<uint32_t>(rb, p.rows);
     // keep the shared memory of one CTA under about 100 KB
     while (rb > 1 && band_smem_bytes(p, rb, bc.pitch) > 100 * 1024) rb--;
+    // single pixels: a thread is busy for longer between its loads and a wide
+    // module gives a CTA fewer than 512 of them, so three CTAs per SM (51
+    // frames of 4 x 185 x 291, paper order: 64 us with two, 57 with three)
+    if (bc.vec == 1)
+        while (rb > 16 && band_smem_bytes(p, rb, bc.pitch) > (200 * 1024) / 3) rb--;
     bc.rb = rb;
     bc.n_bands = (p.rows + rb - 1) / rb;
     bc.fit = true;
