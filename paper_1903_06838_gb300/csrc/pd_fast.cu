@@ -1309,7 +1309,7 @@ cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& cfg, con
     lc.dynamicSmemBytes = smem;
     lc.stream = stream;
     lc.attrs = &attr;
-    lc.numAttrs = early ? 1 : 0;
+    lc.numAttrs = early && n_tiles <= kEarlyWaves * grid ? 1 : 0;
     return cudaLaunchKernelEx(&lc, k, p, raw, frame_base, out, (const BandConfig)bc, n_tiles,
                               (const MultiGain)m);
 }

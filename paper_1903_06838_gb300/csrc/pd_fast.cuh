@@ -36,6 +36,13 @@ struct BandConfig {
     bool ok;
 };
 
+// A call of at most this many waves of persistent CTAs is launched dependent on
+// its common mode (launch_stencil_lean).  That takes 2 to 4 us off any call, but
+// two neighbouring CTAs then often share an SM, and where the occupancy differs
+// from frame to frame both are slow at once: 45 frames of 16 x 352 x 384 at 0.1
+// to 10 % (14 waves) 460 -> 474 us, 120 of 704 x 768 (9 waves) 268 -> 274.
+constexpr uint64_t kEarlyWaves = 4;
+
 // Rows per band of a call over `modules` (frame, module) pairs: at most rb,
 // the default height, which suits calls of many tiles.  A call whose tiles
 // fill the persistent CTAs (`slots`) only a few times ends with a wave that is

@@ -1649,7 +1649,7 @@ cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& cfg, con
     cfg_l.dynamicSmemBytes = smem;
     cfg_l.stream = stream;
     cfg_l.attrs = &attr;
-    cfg_l.numAttrs = early ? 1 : 0;
+    cfg_l.numAttrs = early && n_tiles <= kEarlyWaves * grid ? 1 : 0;
     return cudaLaunchKernelEx(&cfg_l, k, p, raw, frame_base, out, (const LeanConfig)lc, n_tiles,
                               (const CUtensorMap)map, err, mg ? *mg : MultiGain{});
 }

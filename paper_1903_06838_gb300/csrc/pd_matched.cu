@@ -924,7 +924,7 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
         cfg.dynamicSmemBytes = smem;
         cfg.stream = stream;
         cfg.attrs = &attr;
-        cfg.numAttrs = early ? 1 : 0;
+        cfg.numAttrs = early && n_tiles <= kEarlyWaves * grid ? 1 : 0;
         return cudaLaunchKernelEx(&cfg, k, p, bank_dev, raw, frame_base, out, (const BandConfig)bc,
                                   n_tiles);
     }
