@@ -862,7 +862,7 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const MultiGain&
         // A tile with more candidates than threads (a bright one) tests them
         // all first, so that the sums run over its seeds, one in four, with
         // every lane on one (45 frames of 16 x 352 x 384 at 0.1 to 10 %
-        // occupancy: 360 -> 290 us)
+        // occupancy: 360 -> 304 us)
         if (!scan && n_list > nthr) {
             for (uint32_t j = tid; j < n_list; j += nthr) {
                 const float* sc = tile + list[j];

@@ -45,8 +45,9 @@
 // the candidates with a valid feature, so that they keep every lane busy.
 // (Every pixel whose window held any signal was a candidate before: a quarter
 // of all at an occupancy of 0.5 %, each marked with up to eight shared atomics
-// and looked up in the table; 64 frames of 32 x 185 x 388: 556 -> 424 us,
-// with bands of 47 rows in place of 31 and one list of taps for the three sums.)
+// and looked up in the table; 64 frames of 32 x 185 x 388: 556 -> 399 us,
+// with bands of 47 rows in place of 31, one list of taps for the three sums and
+// the common mode of full-height units in registers.)
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
