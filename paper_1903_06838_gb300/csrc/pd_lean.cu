@@ -866,12 +866,14 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const MultiGain&
         if (!scan && n_list > nthr) {
             for (uint32_t j = tid; j < n_list; j += nthr) {
                 const float* sc = tile + list[j];
-                // (a neighbour below the threshold counts as 0, and sp > 0)
+                // (a neighbour below the threshold counts as 0, and sp > 0; so
+                // does a NaN, which fmaxf drops unless all four are NaN: the
+                // tests are written so that they hold for it)
                 const float sp = sc[0];
                 const float q0 = fmaxf(fmaxf(sc[-(int)P - 1], sc[-(int)P]),
                                        fmaxf(sc[-(int)P + 1], sc[-1]));
                 const float q1 = fmaxf(fmaxf(sc[1], sc[P - 1]), fmaxf(sc[P], sc[P + 1]));
-                if ((sp > q0 || q0 <= z) && sp >= q1)
+                if ((sp > q0 || !(q0 > z)) && !(sp < q1))
                     list[lc.list_cap + atomicAdd(&list_n[2], 1u)] = list[j];
             }
             __syncthreads();
