@@ -627,13 +627,17 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const MultiGain&
             out.cm + (size_t)f * (EXTRA == kStacked ? cm_per_frame(p) : p.units_per_frame);
         const float* cmf = cm_frame + (size_t)m * p.units_per_module;
         // kStacked: the module's row terms, and the chunk's four column terms
+        // (the kernel before may still write them when this one starts: ordinary
+        // loads, which the compiler keeps behind wait_previous_kernel, not the
+        // read-only path.  Past L1, by __ldcg, the call of 64 frames of 32 x 185 x
+        // 388 takes 772 us in place of 760: many threads read each term.)
         const float* cmr = cm_frame + p.units_per_frame + (size_t)m * p.rows;
         float2 cc01 = make_float2(0.0f, 0.0f), cc23 = cc01;
         if (EXTRA == kStacked) {
             const float* cmc = cm_frame + p.units_per_frame + (size_t)p.n_modules * p.rows +
                                (size_t)m * p.cols + col;
-            cc01 = make_float2(-__ldg(cmc), -__ldg(cmc + 1));
-            cc23 = make_float2(-__ldg(cmc + 2), -__ldg(cmc + 3));
+            cc01 = make_float2(-cmc[0], -cmc[1]);
+            cc23 = make_float2(-cmc[2], -cmc[3]);
         }
         // stage row of module row r: r + srow0
         const int srow0 =
@@ -748,7 +752,7 @@ __device__ __forceinline__ bool lean_tile(const ChainParams& p, const MultiGain&
                 x.rw = __ldg(reinterpret_cast<const uint2*>(fr + off));
             x.np = __ldg(reinterpret_cast<const float4*>(npm + off));
             x.g = __ldg(reinterpret_cast<const float4*>(gm + off));
-            x.cr = EXTRA == kStacked ? -__ldg(cmr + r) : 0.0f;
+            x.cr = EXTRA == kStacked ? -cmr[r] : 0.0f;
             return x;
         };
 
