@@ -266,11 +266,14 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int i = tid; i < NPOS * 9; i += blockDim.x) s_nb[i] = nb(i / 9, i % 9);
-    // the weight images, and fc_kernel's reads of h2 from the chunk before
+    // the weight images (which prep_weights may still write when this kernel
+    // starts: not by the read-only path), and fc_kernel's reads of h2 from the
+    // chunk before
     wait_previous();
     start_next();
     for (uint32_t i = tid; i < W2_BYTES / 16; i += blockDim.x)
-        reinterpret_cast<uint4*>(sm + WS_W2)[i] = reinterpret_cast<const uint4*>(img + OFF_W2)[i];
+        reinterpret_cast<uint4*>(sm + WS_W2)[i] =
+            __ldcg(reinterpret_cast<const uint4*>(img + OFF_W2) + i);
     fence_async_smem();
     fence_before();
     __syncthreads();

@@ -20,7 +20,9 @@
 // (256 CTAs adding their 9,568 sums to the result atomically took 13 of the
 // step kernel's 35 us.)  Each launch starts while the one before ends
 // (programmatic dependent launch): step_kernel clears its shared memory
-// during prep_kernel.
+// during prep_kernel.  So the images are read by ordinary cached loads and not
+// by the read-only path, whose memory has to stay as it is for the kernel's
+// whole life.
 //
 // Eight hits are 200 (hit, position) rows, thirteen 16-row tiles, and one
 // n-tile of FC3 and its transpose, where the weights are the 16-row operand;
@@ -207,8 +209,8 @@ __device__ __forceinline__ void conv_tiles(uint32_t grid, const uint4* __restric
     const uint32_t r1 = two ? grid + s_row[(mt0 + 8) * 16 + (lane & 15)] + half : r0;
 #pragma unroll
     for (int ks = 0; ks < 18; ks++) {
-        const uint4 b0 = __ldg(img + (ks * 2) * 32 + lane);
-        const uint4 b1 = __ldg(img + (ks * 2 + 1) * 32 + lane);
+        const uint4 b0 = __ldca(img + (ks * 2) * 32 + lane);
+        const uint4 b1 = __ldca(img + (ks * 2 + 1) * 32 + lane);
         const int off = SIGN * tap_off(ks >> 1) * AP + (ks & 1) * 32;
         uint32_t a[4];
         ldsm4(r0 + off, a);
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(THREADS, 2)
 
         // conv1: 16 taps deep
         {
-            const uint4 b0 = __ldg(img + I_W1 + lane), b1 = __ldg(img + I_W1 + 32 + lane);
+            const uint4 b0 = __ldca(img + I_W1 + lane), b1 = __ldca(img + I_W1 + 32 + lane);
             for (int mt = warp; mt < MT; mt += 8) {
                 uint32_t a[4];
                 ldsm4(base + S_XC + (mt * 16 + (lane & 15)) * XP + (lane >> 4) * 16, a);

@@ -19,7 +19,19 @@ WRITTEN = {
     "pd_lean.cu": ["cm_frame", "cmf", "cmr", "cmc", "out.cm"],
     "pd_fast.cu": ["cmf", "cmr", "cmc", "out.cm"],
     "pd_matched.cu": ["cmf", "cmr", "cmc", "out.cm"],
+    # the weight images, activations and gradient sums of the step's kernels
+    "pd_net_train.cu": ["img", "wp", "slices", "dz3", "h2"],
+    "pd_net_tc.cu": ["img", "h2"],
 }
+
+
+def test_weight_images_by_explicit_loads():
+    # a plain load through a const __restrict__ pointer may become one by the
+    # read-only path: the images are read by intrinsics and bulk copies alone
+    for name in ("pd_net_train.cu", "pd_net_tc.cu"):
+        with open(os.path.join(CSRC, name)) as f:
+            text = re.sub(r"//[^\n]*", "", f.read())
+        assert not re.findall(r"const uint4\*>\(img[^()]*\)\[|\bimg\s*\[(?!i\] =)", text)
 
 
 @pytest.mark.parametrize("name", list(WRITTEN))
