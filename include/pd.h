@@ -319,7 +319,9 @@ void pd_destroy(pd_ctx* ctx);
  * keep the current value.  chunk_frames: frames per common-mode/stencil
  * launch pair (a chunk's raw frames are re-read from L2 by the second
  * pass); band_rows: rows per stencil tile (of the default height, calls of few
- * tiles take less); overlap: 1 runs the common mode
+ * tiles take less; PD_EINVAL past what shared memory holds, in the paper's
+ * order the tallest that fits; 0 where the stencil has fixed tiles);
+ * overlap: 1 runs the common mode
  * of the next chunk on a second stream beside the stencil of the current
  * one; two_pass: 0 runs the whole chain as one kernel per (frame, module)
  * where the geometry allows it (common-mode units that are full-height

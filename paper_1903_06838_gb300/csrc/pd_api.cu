@@ -253,6 +253,10 @@ void free_ctx(pd_ctx* c) {
     delete c;
 }
 
+// The band stencil of pd_fast.cu can run this context's calls (in either order;
+// use_band alone: the common mode before gain, as the mixed batch has it).
+bool band_stencil(const pd_ctx* c) { return c->use_band || c->use_band_ag; }
+
 // The one-kernel chain replaces the kernel pair.
 bool fused_on(const pd_ctx* c) { return c->use_fused && !c->two_pass && !c->matched; }
 // (use_fused and use_cm_rows are off for multi-gain contexts: those
@@ -271,7 +275,7 @@ cudaError_t launch_stencil_for(const pd_ctx* c, const uint16_t* fr, uint32_t nf,
         lc.wait_polls = c->wait_polls;
         return pd::launch_stencil_lean(c->params, lc, fr, nf, frame_base, co, c->d_err, s, mg, early);
     }
-    return c->use_band || c->use_band_ag
+    return band_stencil(c)
                ? pd::launch_stencil_band(c->params, c->band_cfg, fr, nf, frame_base, co, s, mg, early)
                : pd::launch_stencil(c->params, fr, nf, frame_base, co, s, mg);
 }
@@ -968,7 +972,7 @@ int pd_get_tuning(const pd_ctx* c, pd_tuning* t) {
     if (!c || !t) return fail(PD_EINVAL, "NULL argument");
     t->chunk_frames = c->chunk_frames;
     const bool lean = c->use_lean && (c->kernels == 1 || c->kernels == 3) && !c->matched;
-    t->band_rows = lean ? c->lean_cfg.rb : c->use_band ? c->band_cfg.rb : 0;
+    t->band_rows = lean ? c->lean_cfg.rb : band_stencil(c) ? c->band_cfg.rb : 0;
     t->overlap = c->overlap;
     t->two_pass = c->use_fused && !c->matched ? c->two_pass : 1;
     t->kernels = c->use_lean || c->use_bank || c->use_row_codes ? (c->kernels == 3 && !c->use_queue ? 1u : c->kernels)
@@ -987,10 +991,14 @@ int pd_set_tuning(pd_ctx* c, const pd_tuning* t) {
             return fail(PD_EINVAL, "band too tall for shared memory");
         c->lean_cfg = lc;
     }
-    if (t->band_rows && c->use_band) {
-        const uint32_t rb = std::min(t->band_rows, c->params.rows);
-        if (pd::band_smem_bytes(c->params, rb, c->band_cfg.pitch) > 200 * 1024)
-            return fail(PD_EINVAL, "band too tall for shared memory");
+    if (t->band_rows && band_stencil(c)) {
+        uint32_t rb = std::min(t->band_rows, c->params.rows);
+        const auto fits = [&] {
+            return pd::band_smem_bytes(c->params, rb, c->band_cfg.pitch) <= 200 * 1024;
+        };
+        // the paper's order took any height while it had no bands
+        while (c->use_band_ag && rb > 1 && !fits()) rb--;
+        if (!fits()) return fail(PD_EINVAL, "band too tall for shared memory");
         c->band_cfg.rb = rb;
         c->band_cfg.fit = rb == pd::make_band_config(c->params).rb;
         c->band_cfg.n_bands = (c->params.rows + rb - 1) / rb;
@@ -1421,7 +1429,7 @@ int pd_autotune(pd_ctx* c, const uint16_t* frames_dev, uint32_t n_frames, pd_tun
         for (uint32_t k : kopts) {
             std::vector<uint32_t> bands = {0};
             if (!c->matched && k == 1 && c->use_lean) bands = band_set(lean_rb0);
-            else if (!c->matched && c->use_band) bands = band_set(band_rb0);
+            else if (!c->matched && band_stencil(c)) bands = band_set(band_rb0);
             for (uint32_t cf : chunks)
                 for (uint32_t bd : bands)
                     for (uint32_t ov : {1u, 0u}) cands.push_back(pd_tuning{cf, bd, ov, 1, k});
