@@ -138,13 +138,14 @@ __device__ __forceinline__ UnitAt unit_at(const ChainParams& p, uint32_t f, uint
 // position advances with a carry instead of a division.  V = 2 needs even
 // columns and unit widths (4- and 8-byte loads).  f(v) sees every pixel of the
 // unit and, at the end, NaN in the place of pixels past it; after() runs every
-// 4 V pixels.
+// kSweepSteps V pixels.
+constexpr int kSweepSteps = 4;
 template <int V, bool AG, class F, class G>
 __device__ __forceinline__ void sweep_unit(const ChainParams& p, const uint16_t* __restrict__ rw,
                                            const float* __restrict__ np_,
                                            const float* __restrict__ ig_, uint32_t t,
                                            uint32_t stride, F f, G after) {
-    constexpr int U = 4;
+    constexpr int U = kSweepSteps;
     const uint32_t W = p.unit_cols / V, n = p.unit_rows * W;
     const uint32_t dr = stride / W, dc = stride - dr * W;
     uint32_t c = t % W, off = t / W * p.cols + c * V;
@@ -187,12 +188,14 @@ __device__ __forceinline__ void sweep_unit(const ChainParams& p, const uint16_t*
 }
 
 // One pass where the context's pedestals allow it (p.mean_frac = g >= 0): every
-// selected d is then a whole number of 2^-g below 2^26 of them (see
+// selected d is then a whole number of 2^-g below 2^26 (kFixedBits) of them (see
 // mean_frac_bits), a grid the definition's 2^(E-38) always divides, so the
 // integers can be added without knowing M, and the unit is read once.
+constexpr int kFixedBits = 26;
 struct FixedAcc {
     uint32_t n0 = 0;
-    int part = 0;         // of at most 32 values
+    int part = 0;         // of the kSweepSteps V <= 8 values between two flushes
+    static_assert(((2ll * kSweepSteps) << kFixedBits) < (1ll << 31), "part in 32 bits");
     long long total = 0;
     __device__ __forceinline__ void add(float d, float cut, float scale) {
         const bool sel = d < cut;
@@ -679,7 +682,7 @@ int mean_frac_bits(const ChainParams& p, const float* pedestal) {
         g = std::max(g, 150 - std::max(e, 1) - __builtin_ctz(mant));
         if (g > 24) return -1;
     }
-    return ldexpf(most, g) < 67108864.0f ? g : -1;
+    return ldexpf(most, g) < (float)(1 << kFixedBits) ? g : -1;
 }
 
 cudaError_t launch_cm_mean(const ChainParams& p, const uint16_t* raw, uint32_t n_frames,
