@@ -337,6 +337,9 @@ size_t rows_cols_smem_bytes(const ChainParams& p) {
     return ((size_t)p.units_per_module + p.rows + 4 * (size_t)p.cols) * 4;
 }
 
+// NP: column pairs a lane holds, one per 64 columns.  Up to seven, a row's loads,
+// values and column sums fit 128 registers and two CTAs an SM; more take 148 to
+// 254 and one CTA (none spills).
 template <int NP>
 __global__ void __launch_bounds__(kMeanThreads, NP <= 7 ? 2 : 1)
     mean_rows_cols_kernel(ChainParams p, const uint16_t* __restrict__ raw,
@@ -649,12 +652,18 @@ bool rows_cols_ok(const ChainParams& p) {
 
 void launch_rows_cols(const ChainParams& p, const uint16_t* fr, float* cm, uint32_t nf,
                       cudaStream_t s) {
-    const uint32_t np = (p.cols + 63) / 64;
-    auto k = np <= 3    ? mean_rows_cols_kernel<3>
-             : np <= 6  ? mean_rows_cols_kernel<6>
-             : np <= 7  ? mean_rows_cols_kernel<7>
-             : np <= 12 ? mean_rows_cols_kernel<12>
-                        : mean_rows_cols_kernel<16>;
+    // an instance for every number of pairs, so that no lane sums pairs past the
+    // row's end (the call of 60 frames of 4 x 400 rows, against instances for 3, 6,
+    // 7, 12 and 16 pairs: 64 columns 73 -> 60 us, 256 149 -> 131, 512 313 -> 264)
+    using Kernel = decltype(&mean_rows_cols_kernel<1>);
+    constexpr Kernel by_groups[] = {
+        mean_rows_cols_kernel<1>,  mean_rows_cols_kernel<2>,  mean_rows_cols_kernel<3>,
+        mean_rows_cols_kernel<4>,  mean_rows_cols_kernel<5>,  mean_rows_cols_kernel<6>,
+        mean_rows_cols_kernel<7>,  mean_rows_cols_kernel<8>,  mean_rows_cols_kernel<9>,
+        mean_rows_cols_kernel<10>, mean_rows_cols_kernel<11>, mean_rows_cols_kernel<12>,
+        mean_rows_cols_kernel<13>, mean_rows_cols_kernel<14>, mean_rows_cols_kernel<15>,
+        mean_rows_cols_kernel<16>};
+    const Kernel k = by_groups[(p.cols + 63) / 64 - 1];
     k<<<nf * p.n_modules, kMeanThreads, rows_cols_smem_bytes(p), s>>>(p, fr, cm);
 }
 }  // namespace
