@@ -1251,20 +1251,24 @@ size_t band_smem_bytes(const ChainParams& p, uint32_t rb, uint32_t pitch) {
            (size_t)(rb + 1) * ((p.cols + 31) / 32) * 4;     // seed bitmap
 }
 
+static int band_ctas_per_sm(const ChainParams& p, const BandConfig& bc) {
+    const size_t smem = band_smem_bytes(p, bc.rb, bc.pitch);
+    return (int)std::max<size_t>(1, std::min<size_t>((200 * 1024) / smem, 4));
+}
+
+uint32_t band_call_rows(const ChainParams& p, const BandConfig& bc, uint32_t n_frames, int sms) {
+    if (!bc.fit) return bc.rb;
+    return fit_band_rows(p.rows, bc.rb, bc.ty, (uint64_t)n_frames * p.n_modules,
+                         (uint64_t)sms * band_ctas_per_sm(p, bc));
+}
+
 cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& cfg, const uint16_t* raw,
                                 uint32_t n_frames, uint32_t frame_base, const CallOut& out,
                                 cudaStream_t stream, const MultiGain* mg, bool early) {
     if (n_frames == 0) return cudaSuccess;
     BandConfig bc = cfg;
-    const auto ctas_per_sm = [&] {
-        const size_t smem = band_smem_bytes(p, bc.rb, bc.pitch);
-        return (int)std::max<size_t>(1, std::min<size_t>((200 * 1024) / smem, 4));
-    };
-    if (bc.fit) {
-        bc.rb = fit_band_rows(p.rows, bc.rb, bc.ty, (uint64_t)n_frames * p.n_modules,
-                              (uint64_t)device_sm_count() * ctas_per_sm());
-        bc.n_bands = (p.rows + bc.rb - 1) / bc.rb;
-    }
+    bc.rb = band_call_rows(p, cfg, n_frames, device_sm_count());
+    bc.n_bands = (p.rows + bc.rb - 1) / bc.rb;
     const unsigned long long n_tiles = (unsigned long long)n_frames * p.n_modules * bc.n_bands;
     if (mg && (bc.vec != 4 || cm_after_gain(p))) return cudaErrorInvalidValue;
     int dev = 0;
@@ -1285,7 +1289,7 @@ cudaError_t launch_stencil_band(const ChainParams& p, const BandConfig& cfg, con
     }
     const size_t smem = band_smem_bytes(p, bc.rb, bc.pitch);
     const unsigned threads = bc.tx * bc.ty;
-    unsigned long long grid = (unsigned long long)device_sm_count() * ctas_per_sm();
+    unsigned long long grid = (unsigned long long)device_sm_count() * band_ctas_per_sm(p, bc);
     if (grid > n_tiles) grid = n_tiles;
     const bool st = cm_kind(p) == PD_CM_MEAN_STACKED;
     const MultiGain m = mg ? *mg : MultiGain{};

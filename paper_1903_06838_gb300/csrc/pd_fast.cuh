@@ -117,6 +117,8 @@ cudaError_t launch_cm_rows(const ChainParams& p, const uint16_t* raw, uint32_t n
 
 BandConfig make_band_config(const ChainParams& p);
 size_t band_smem_bytes(const ChainParams& p, uint32_t rb, uint32_t pitch);
+// Rows per band of a call on sms SMs (fit_band_rows where bc.fit).
+uint32_t band_call_rows(const ChainParams& p, const BandConfig& bc, uint32_t n_frames, int sms);
 // mg: auto-ranging words (four-pixel chunks and the median or no common
 // mode only), or NULL.  early: the launch before in the stream is this call's
 // common mode.

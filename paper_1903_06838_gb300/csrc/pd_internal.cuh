@@ -168,6 +168,8 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
                            const uint16_t* raw, uint32_t n_frames, uint32_t frame_base,
                            const CallOut& out, cudaStream_t stream,
                            const MultiGain* mg = nullptr, bool early = false);
+// Rows per band of a call on sms SMs, 0 where the tile kernel runs.
+uint32_t matched_call_rows(const ChainParams& p, uint32_t n_frames, int sms);
 // The paper's mean estimator, one stage or three stacked (pd_cm_mean.cu).
 int mean_frac_bits(const ChainParams& p, const float* pedestal);
 cudaError_t launch_cm_mean(const ChainParams& p, const uint16_t* raw, uint32_t n_frames,

@@ -1541,6 +1541,15 @@ LeanConfig make_lean_config(const ChainParams& p, uint32_t rb, bool multigain) {
     return lc;
 }
 
+uint32_t lean_call_rows(const ChainParams& p, const LeanConfig& lc, uint32_t n_frames, int sms) {
+    if (!lc.fit) return lc.rb;
+    const uint64_t slots =
+        (uint64_t)sms * (lc.ctas_per_sm                          ? lc.ctas_per_sm
+                         : lean_smem_bytes(p, lc) <= kLeanSmemTwo ? 2u
+                                                                  : 1u);
+    return fit_band_rows(p.rows, lc.rb, lc.ty, (uint64_t)n_frames * p.n_modules, slots);
+}
+
 size_t lean_smem_bytes(const ChainParams& p, const LeanConfig& lc) {
     const size_t stage = staged(lc) ? ((size_t)lc.stage_bp * lc.stage_g * 16 + 127) / 128 * 128 : 0;
     return stage + (size_t)(lc.rb + 2) * lc.pitch * 4 + 2 * (size_t)p.hist_bins * 4 +
@@ -1571,14 +1580,9 @@ cudaError_t launch_stencil_lean(const ChainParams& p, const LeanConfig& cfg, con
                                 uint32_t* err, cudaStream_t stream, const MultiGain* mg, bool early) {
     if (n_frames == 0) return cudaSuccess;
     LeanConfig lc = cfg;
-    if (lc.fit) {
-        const uint64_t slots = (uint64_t)device_sm_count() *
-                               (lc.ctas_per_sm ? lc.ctas_per_sm
-                                : lean_smem_bytes(p, lc) <= kLeanSmemTwo ? 2u : 1u);
-        lc.rb = fit_band_rows(p.rows, lc.rb, lc.ty, (uint64_t)n_frames * p.n_modules, slots);
-        lc.n_bands = (p.rows + lc.rb - 1) / lc.rb;
-        set_stage_periods(lc);
-    }
+    lc.rb = lean_call_rows(p, cfg, n_frames, device_sm_count());
+    lc.n_bands = (p.rows + lc.rb - 1) / lc.rb;
+    set_stage_periods(lc);
     const unsigned long long n_tiles = (unsigned long long)n_frames * p.n_modules * lc.n_bands;
     int dev = 0;
     cudaGetDevice(&dev);

@@ -103,6 +103,8 @@ struct LeanConfig {
 // multigain: the words are auto-ranging ones.
 LeanConfig make_lean_config(const ChainParams& p, uint32_t rb = 0, bool multigain = false);
 size_t lean_smem_bytes(const ChainParams& p, const LeanConfig& lc);
+// Rows per band of a call on sms SMs (fit_band_rows where lc.fit).
+uint32_t lean_call_rows(const ChainParams& p, const LeanConfig& lc, uint32_t n_frames, int sms);
 // raw: 16-byte aligned.  err: context error word (bit 1: a bounded wait
 // for a staged copy gave up).  mg: auto-ranging words, or NULL.  early: the
 // launch before in the stream is this call's common mode.

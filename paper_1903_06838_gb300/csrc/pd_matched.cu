@@ -879,6 +879,22 @@ static bool matched_band_config(const ChainParams& p, BandConfig* out) {
     return true;
 }
 
+static int matched_ctas_per_sm(const ChainParams& p, const BandConfig& bc) {
+    const size_t per_cta = band_smem(p, bc.rb, bc.pitch) + sizeof(MatchedBank) + 1024;
+    return (int)std::max<size_t>(1, std::min<size_t>((228 * 1024) / per_cta, 2));
+}
+
+static uint32_t band_rows_of(const ChainParams& p, const BandConfig& bc, uint32_t n_frames,
+                             int sms) {
+    return fit_band_rows(p.rows, bc.rb, bc.ty, (uint64_t)n_frames * p.n_modules,
+                         (uint64_t)sms * matched_ctas_per_sm(p, bc));
+}
+
+uint32_t matched_call_rows(const ChainParams& p, uint32_t n_frames, int sms) {
+    BandConfig bc;
+    return matched_band_config(p, &bc) ? band_rows_of(p, bc, n_frames, sms) : 0;
+}
+
 static int g_attr_dev_mband = -1;
 
 cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
@@ -888,12 +904,7 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
     BandConfig bc;
     if (!mg && matched_band_config(p, &bc)) {
         if (n_frames == 0) return cudaSuccess;
-        const auto ctas_per_sm = [&] {
-            const size_t per_cta = band_smem(p, bc.rb, bc.pitch) + sizeof(MatchedBank) + 1024;
-            return (int)std::max<size_t>(1, std::min<size_t>((228 * 1024) / per_cta, 2));
-        };
-        bc.rb = fit_band_rows(p.rows, bc.rb, bc.ty, (uint64_t)n_frames * p.n_modules,
-                              (uint64_t)device_sm_count() * ctas_per_sm());
+        bc.rb = band_rows_of(p, bc, n_frames, device_sm_count());
         bc.n_bands = (p.rows + bc.rb - 1) / bc.rb;
         const unsigned long long n_tiles =
             (unsigned long long)n_frames * p.n_modules * bc.n_bands;
@@ -909,7 +920,8 @@ cudaError_t launch_matched(const ChainParams& p, const MatchedBank* bank_dev,
             g_attr_dev_mband = dev;
         }
         const size_t smem = band_smem(p, bc.rb, bc.pitch);
-        unsigned long long grid = (unsigned long long)device_sm_count() * ctas_per_sm();
+        unsigned long long grid =
+            (unsigned long long)device_sm_count() * matched_ctas_per_sm(p, bc);
         if (grid > n_tiles) grid = n_tiles;
         const unsigned threads = bc.tx * bc.ty;
         const bool st = cm_kind(p) == PD_CM_MEAN_STACKED, col = p.unit_rows == p.rows;
