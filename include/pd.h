@@ -320,7 +320,9 @@ void pd_destroy(pd_ctx* ctx);
  * launch pair (a chunk's raw frames are re-read from L2 by the second
  * pass); band_rows: rows per stencil tile (of the default height, calls of few
  * tiles take less; PD_EINVAL past what shared memory holds, in the paper's
- * order the tallest that fits; 0 where the stencil has fixed tiles);
+ * order the tallest that fits, and the lean stencil of the stacked mean and of
+ * auto-ranging words takes its tallest for heights that only the earlier one
+ * holds; 0 where the stencil has fixed tiles);
  * overlap: 1 runs the common mode
  * of the next chunk on a second stream beside the stencil of the current
  * one; two_pass: 0 runs the whole chain as one kernel per (frame, module)

@@ -985,23 +985,28 @@ int pd_set_tuning(pd_ctx* c, const pd_tuning* t) {
     if (t->chunk_frames) c->chunk_frames = t->chunk_frames;
     if (t->kernels > 3) return fail(PD_EINVAL, "kernels is 0, 1, 2 or 3");
     if (t->kernels) c->kernels = t->kernels;
-    if (t->band_rows && c->use_lean) {
-        const pd::LeanConfig lc = pd::make_lean_config(c->params, t->band_rows, c->multigain);
-        if (!lc.ok || lc.rb != std::min(t->band_rows, c->params.rows))
+    if (t->band_rows) {
+        const uint32_t want = std::min(t->band_rows, c->params.rows);
+        const pd::LeanConfig lc =
+            c->use_lean ? pd::make_lean_config(c->params, want, c->multigain) : c->lean_cfg;
+        // The stacked mean and auto-ranging words ran the band stencil, which
+        // holds taller bands: their lean stencil takes the tallest it holds.
+        const bool cut = c->multigain || pd::cm_kind(c->params) == PD_CM_MEAN_STACKED;
+        if (c->use_lean && (!lc.ok || (lc.rb != want && !cut)))
             return fail(PD_EINVAL, "band too tall for shared memory");
+        if (band_stencil(c)) {
+            uint32_t rb = want;
+            const auto fits = [&] {
+                return pd::band_smem_bytes(c->params, rb, c->band_cfg.pitch) <= 200 * 1024;
+            };
+            // the paper's order took any height while it had no bands
+            while (c->use_band_ag && rb > 1 && !fits()) rb--;
+            if (!fits()) return fail(PD_EINVAL, "band too tall for shared memory");
+            c->band_cfg.rb = rb;
+            c->band_cfg.fit = rb == pd::make_band_config(c->params).rb;
+            c->band_cfg.n_bands = (c->params.rows + rb - 1) / rb;
+        }
         c->lean_cfg = lc;
-    }
-    if (t->band_rows && band_stencil(c)) {
-        uint32_t rb = std::min(t->band_rows, c->params.rows);
-        const auto fits = [&] {
-            return pd::band_smem_bytes(c->params, rb, c->band_cfg.pitch) <= 200 * 1024;
-        };
-        // the paper's order took any height while it had no bands
-        while (c->use_band_ag && rb > 1 && !fits()) rb--;
-        if (!fits()) return fail(PD_EINVAL, "band too tall for shared memory");
-        c->band_cfg.rb = rb;
-        c->band_cfg.fit = rb == pd::make_band_config(c->params).rb;
-        c->band_cfg.n_bands = (c->params.rows + rb - 1) / rb;
     }
     c->overlap = t->overlap ? 1 : 0;
     c->two_pass = t->two_pass ? 1 : 0;
