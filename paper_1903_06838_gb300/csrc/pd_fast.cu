@@ -871,7 +871,7 @@ __device__ void stencil_band_run(const ChainParams& p, const uint16_t* __restric
                 if (word) sbits[rl * WPR + w] = 0;
                 rc = rl << 16 | 32 * w;
             }
-            const unsigned wm = __activemask();
+            const unsigned wm = warp_lanes();
             const uint32_t cnt = (uint32_t)__popc(word);
             uint32_t incl = cnt;
 #pragma unroll

@@ -627,7 +627,7 @@ __global__ void __launch_bounds__(kBandThreads, 2)
                 word &= ~over;
                 if (C - x0 < 32) word &= 0xFFFFFFFFu >> (32 - (C - x0));
             }
-            const unsigned wm = __activemask();
+            const unsigned wm = warp_lanes();
             const uint32_t cnt = (uint32_t)__popc(word);
             uint32_t incl = cnt;
 #pragma unroll
