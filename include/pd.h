@@ -211,8 +211,8 @@ int pd_create(const pd_geometry* geometry, const float* pedestal_host,
  * others; a stage >= n_gains marks a bad pixel, e = 0.  Everything after
  * the energy (zeroing, charge summing or matched filters, summaries) is
  * unchanged.  1 <= n_gains <= PD_MAX_GAINS, 1 <= gain_shift <= 15, cm_mode
- * PD_CM_MEDIAN or PD_CM_NONE; such contexts use the generic kernels (no
- * one-kernel chain, no mixed batch launch).  masked_pixels counts stage 0. */
+ * PD_CM_MEDIAN or PD_CM_NONE; such contexts have no one-kernel
+ * chain and no mixed batch launch.  masked_pixels counts stage 0. */
 #define PD_MAX_GAINS 4u
 int pd_create_multigain(const pd_geometry* geometry, uint32_t n_gains, uint32_t gain_shift,
                         const float* pedestal_host, const float* gain_host,
@@ -332,11 +332,11 @@ void pd_destroy(pd_ctx* ctx);
  * default; pd_get_tuning reports 1 when the one-kernel form is not
  * available).
  * kernels: 1 runs the lean pair where the context allows it (the default:
- * the integer-coded bank median for units of 4096+ pixels whose pedestals
- * keep d = raw - pedestal exact inside the common-mode window, and the lean
- * band stencil for columns a multiple of 4, single-gain words, the median,
- * no or the one-stage mean common mode, subtracted before gain); 2 runs the
- * earlier kernel pair (pd_get_tuning reports 2 when the lean pair is not
+ * the integer-coded medians of units of 4096+ pixels and of one-row units of
+ * up to 512 pixels in fours, where the pedestals keep d = raw - pedestal exact
+ * inside the common-mode window, and the lean band stencil for columns a
+ * multiple of 4 and a common mode subtracted before gain); 2 runs the earlier
+ * kernel pair (pd_get_tuning reports 2 when no kernel of the lean pair is
  * available); 3 runs the lean pair as one persistent launch per call over a
  * work queue (bank medians of a few frames, then the stencil tiles of the
  * frames before them, so raw is re-read from L2; column-bank units, no

@@ -523,7 +523,7 @@ constexpr uint32_t kLeanThreads = 512;
 
 // What a lean stencil instance handles beside the plain energies (64 frames
 // of 32 x 185 x 388, against the band stencil of pd_fast.cu that ran them
-// before: stacked 362 -> 272 us, auto-ranging 448 -> 371 us).
+// before: stacked 362 -> 261 us, auto-ranging 448 -> 340 us).
 constexpr int kPlain = 0;
 constexpr int kStacked = 1;    // the stacked mean's module-row and module-column terms
 constexpr int kMultiGain = 2;  // auto-ranging words

@@ -47,7 +47,13 @@
 // of all at an occupancy of 0.5 %, each marked with up to eight shared atomics
 // and looked up in the table; 64 frames of 32 x 185 x 388: 556 -> 399 us,
 // with bands of 47 rows in place of 31, one list of taps for the three sums and
-// the common mode of full-height units in registers.)
+// the common mode of full-height units in registers.  64 registers, so that two
+// CTAs fit an SM, and 88 to 96 bytes of spills.)
+// That holds while a tile's candidates fit kMbCap: a 47 x 388 tile has some 630
+// at an occupancy of 0.5 %, 1200 at 1 %, 2200 at 2 %.  Past it every own pixel of
+// the tile is tested, which costs 3.5 times as much; the call of 64 frames, before
+// and now: 0.2 % 696 -> 595 us, 1 % 1076 -> 667 (the longer list of any signal in
+// the window overflowed there), 1.5 % 733, 2 % 2123 -> 2017, 5 % 2442 -> 2387.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
