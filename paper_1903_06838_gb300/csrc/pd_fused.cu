@@ -657,7 +657,12 @@ cudaError_t launch_fused(const ChainParams& p, const FusedConfig& fc, const uint
         if (e != cudaSuccess) return e;
         g_attr_dev_fused = dev;
     }
-    const unsigned threads = (fc.tx * fc.ty + 31) / 32 * 32;
+    // (a warp locates each unit's median bin: a narrow module of two banks has
+    // fewer threads of its own than two warps)
+    const unsigned warps =
+        std::max((fc.tx * fc.ty + 31) / 32,
+                 cm_kind(p) == PD_CM_MEDIAN ? p.units_per_row : 1u);
+    const unsigned threads = 32 * warps;
     return threads <= 320
                ? launch_fused_t<320>(p, fc, raw, n_frames, frame_base, out, stream, threads, items)
                : launch_fused_t<512>(p, fc, raw, n_frames, frame_base, out, stream, threads, items);
