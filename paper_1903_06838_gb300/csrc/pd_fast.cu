@@ -1014,6 +1014,23 @@ __device__ __forceinline__ uint32_t find_item(const BatchItem* items, uint32_t n
     return lo;
 }
 
+// The selections of the launch that holds every kind, as calls.  Inlined there
+// side by side, a unit's whole-unit selection left the first warp of the block
+// apart, and its parts arrived at the barriers of the block's next units one by
+// one: generic units after such a large one came out wrong.  (The source has no
+// barrier that a part of a warp reaches; with barriers that allow a split warp
+// in the selections, or with calls, every unit is right.)
+template <int VEC>
+__device__ __noinline__ void big_task(const BatchItem& it, uint32_t local, uint32_t* smem,
+                                      CmBigShared& big) {
+    cm_big_unit<VEC>(it.p, it.raw, it.out.cm, it.cm_cfg, local, smem, big);
+}
+template <bool KEYS_IN_SMEM>
+__device__ __noinline__ void generic_task(const BatchItem& it, uint32_t local, uint32_t* smem,
+                                          generic_cm::Shared& gen) {
+    generic_cm::unit<KEYS_IN_SMEM>(it.p, it.raw, it.out.cm, local, smem, gen);
+}
+
 // ALL_KINDS false: every item's common mode is a bank with pairs of
 // pixels (kind 0) or rows (kind 4), the usual mix; the kernel then carries
 // only those two paths (fewer registers).
@@ -1040,10 +1057,10 @@ __global__ void __launch_bounds__(512, 2)
             cm_big_unit<2>(it.p, it.raw, it.out.cm, it.cm_cfg, local, smem, big);
         } else {
             switch (it.cm_kind) {
-                case 0: cm_big_unit<2>(it.p, it.raw, it.out.cm, it.cm_cfg, local, smem, big); break;
-                case 1: cm_big_unit<1>(it.p, it.raw, it.out.cm, it.cm_cfg, local, smem, big); break;
-                case 2: generic_cm::unit<true>(it.p, it.raw, it.out.cm, local, smem, gen); break;
-                default: generic_cm::unit<false>(it.p, it.raw, it.out.cm, local, smem, gen); break;
+                case 0: big_task<2>(it, local, smem, big); break;
+                case 1: big_task<1>(it, local, smem, big); break;
+                case 2: generic_task<true>(it, local, smem, gen); break;
+                default: generic_task<false>(it, local, smem, gen); break;
             }
         }
         __syncthreads();  // shared memory is reused by the next task

@@ -16,8 +16,9 @@
 //
 // The bank is compiled on the host into lists of the nonzero taps.  Skipping
 // a zero tap is exact for finite signals (1 / gain overflows for gains below
-// 2.9e-39 ADU/keV, where an infinite signal times 0 would be NaN): its term is +-0, and a sum that starts at +0.0f is
-// never -0 (x + (-x) rounds to +0), so adding +-0 never changes it.  For the
+// 2.9e-39 ADU/keV, where an infinite signal times 0 would be NaN): its term is
+// +-0, and a sum that starts at +0.0f is never -0 (x + (-x) rounds to +0), so
+// adding +-0 never changes it.  For the
 // same reason a pixel whose 4 x 5 window holds no signal has every Size,
 // Overflow and Droplet equal to 0, so its energy is 0 and it is skipped.
 //
